@@ -94,7 +94,7 @@ struct Workspace {
   Buf sidx[2], srank[2], scount;
   Buf ckeys, ckeys_alt, ccount, sorttmp;
   Buf piv_key, piv_coef, r_off, r_len, reduced, claim, reduce, heavy, lists;
-  Buf r_key, r_coef, r_top;
+  Buf r_key, r_coef, r_top, wide;
   Buf tkeys[2], tvals[2];
   Buf amk[2];  // apparent-pair maps of dimensions d and d - 1 ((key, value) pairs)
   Buf bars, bars_alt, bk0, bk1, bp0, bp1, bartmp, nbars;
@@ -678,20 +678,21 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
     // a generated coboundary holds at most max_deg entries (sorted in a power-of-two buffer)
     const int blocks = M ? reduction_blocks(a, M) : 1;
     if (blocks < 1) return RIPS_ERR_CUDA;
+    CR(ensure(w.wide, wide_ctx_bytes(blocks)));
     uint32_t slice = 32;
     while (slice < max_deg + 1) slice <<= 1;
-    // The arena holds every run a reduction writes (generated coboundaries,
-    // merges, stored columns), which long chains make large; an arena that
-    // proves too small costs a rerun of the dimension with 8x the room, so a
-    // first call starts at up to 2^30 entries (12 GB) when the device has 16x
-    // that free (the workspace keeps it for later calls).
+    // The arena holds the working columns' tables and lists and the stored
+    // columns; an arena that proves too small costs a rerun of the dimension with
+    // 8x the room, so a first call starts at 2^25 entries (400 MB), or for many
+    // columns at up to 2^30 (12 GB), when the device has 16x that free (the
+    // workspace keeps it for later calls).
     size_t rcap = lim.arena_entries ? (size_t)lim.arena_entries
                                     : std::max<size_t>(w.r_cap, std::max<size_t>(16 * (size_t)M, (size_t)1 << 22));
-    if (!lim.arena_entries && M > 4096) {
+    const size_t first = (size_t)1 << (M > 4096 ? 30 : 25);
+    if (!lim.arena_entries && M && rcap < first) {
       size_t free_b = 0, total_b = 0;
       if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
-        const size_t roomy = std::min<size_t>((size_t)1 << 30, free_b / 16 / 12);
-        rcap = std::max(rcap, roomy);
+        rcap = std::max(rcap, std::min<size_t>(first, free_b / 16 / 12));
       } else {
         cudaGetLastError();
       }
@@ -731,8 +732,7 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       rs.max_chain = counts + 7;
       rs.heartbeat = counts + 12;
       rs.added = P<unsigned long long>(w.lists) + 7;
-      rs.help = (HelpBoard*)(P<unsigned char>(w.lists) + 256);
-      rs.idle = counts + 4;
+      rs.wide = P<WideCtx>(w.wide);
       rs.barrier_ns = lim.barrier_wait_ns ? lim.barrier_wait_ns : 30ull * 1000 * 1000 * 1000;
       rs.chain_ns = lim.chain_ns ? lim.chain_ns : 600ull * 1000 * 1000 * 1000;
       rs.err = P<uint32_t>(w.err);
@@ -1127,7 +1127,7 @@ void release_plan(PlanState& pl) {
                 &w.escan, &w.erank, &w.rvalue, &w.R, &w.deg, &w.nbr, &w.eu, &w.ev, &w.comp, &w.best, &w.parent,
                 &w.gtop, &w.inforest, &w.fpos, &w.nf, &w.sidx[0], &w.sidx[1], &w.srank[0], &w.srank[1],
                 &w.scount, &w.ckeys, &w.ckeys_alt, &w.ccount, &w.sorttmp, &w.piv_key, &w.piv_coef, &w.r_off,
-                &w.r_len, &w.reduced, &w.claim, &w.reduce, &w.heavy, &w.lists, &w.r_key, &w.r_coef, &w.r_top,
+                &w.r_len, &w.reduced, &w.claim, &w.reduce, &w.heavy, &w.lists, &w.r_key, &w.r_coef, &w.r_top, &w.wide,
                 &w.tkeys[0], &w.tkeys[1], &w.tvals[0], &w.tvals[1], &w.amk[0], &w.amk[1],
                 &w.bars, &w.bars_alt, &w.bk0, &w.bk1, &w.bp0, &w.bp1, &w.bartmp, &w.nbars, &w.stats,
                 &w.bwd_bars, &w.bwd_off, &w.cdist, &w.clouds, &w.tileoff, &w.vcloud, &w.ccounts, &pl.clouds0,
@@ -1277,6 +1277,7 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   a.vbits = packed_vertex_bits(pl.n_max, 1);
   pl.blocks = reduction_blocks(a, (uint32_t)E);
   if (pl.blocks < 1) return RIPS_ERR_CUDA;
+  CR(ensure(w.wide, wide_ctx_bytes(pl.blocks)));
   return RIPS_OK;
 }
 
@@ -1371,8 +1372,7 @@ int plan_run(PlanState& pl, const float* d_points, cudaStream_t s) {
   rs.max_chain = counts + 7;
   rs.heartbeat = counts + 12;
   rs.added = P<unsigned long long>(w.lists) + 7;
-  rs.help = (HelpBoard*)(P<unsigned char>(w.lists) + 256);
-  rs.idle = counts + 4;
+  rs.wide = P<WideCtx>(w.wide);
   const rips_limits_t lim = current_limits();
   rs.barrier_ns = lim.barrier_wait_ns ? lim.barrier_wait_ns : 30ull * 1000 * 1000 * 1000;
   rs.chain_ns = lim.chain_ns ? lim.chain_ns : 600ull * 1000 * 1000 * 1000;

@@ -207,9 +207,9 @@ struct DimArgs {
   uint32_t opts;                   // RIPS_OPT_* switches (rips_set_options)
 };
 
-struct HelpBoard;  // rips_dim.cu
+struct WideCtx;  // rips_wide.cuh
 // bytes of the reduction's control block: counters and cursors in the first
-// 256, the help board after them (zeroed together before every launch)
+// 256, the lists of suspended columns after them (zeroed before every launch)
 constexpr size_t LISTS_BYTES = 16384;
 
 // Reduction state (device pointers) shared by the reduction kernels
@@ -244,11 +244,7 @@ struct RedState {
   uint32_t* max_chain;            // longest chain of additions (profiling)
   unsigned* heartbeat;            // bumped while chains of additions make progress
   unsigned long long* added;      // entries of the columns added (profiling)
-  // board through which a block with a large run merge hands chunks of it to
-  // blocks waiting at the grid barrier (zeroed before the launch; null: none),
-  // and the number of blocks waiting there
-  struct HelpBoard* help;
-  const unsigned* idle;
+  WideCtx* wide;                  // one context a block for the columns it suspends (wide_ctx_bytes)
   unsigned long long barrier_ns;  // grid-barrier wait without progress before giving up
   unsigned long long chain_ns;    // one chain of additions before giving up
   uint32_t* err;
@@ -279,6 +275,8 @@ cudaError_t launch_test(const DimArgs& a, const uint64_t* sidx, const uint32_t* 
                         const uint8_t* cleared_flag, const uint64_t* prev_keys, uint64_t prev_mask,
                         uint64_t* col_keys, uint32_t* ncols, uint32_t col_cap, unsigned long long* stats,
                         int stats_stride, cudaStream_t st);
+// bytes of the contexts (RedState::wide) of a reduction by `blocks` blocks
+size_t wide_ctx_bytes(int blocks);
 // blocks of the cooperative reduction launch (all co-resident), -1 on error
 int reduction_blocks(const DimArgs& a, uint32_t ncols);
 // ctl: 8 zeroed uint32 (see reduce_persistent_kernel); ctl[6] receives the rounds
