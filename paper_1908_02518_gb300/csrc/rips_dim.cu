@@ -498,6 +498,17 @@ __device__ __forceinline__ uint64_t table_key(const DimArgs& a, uint32_t cloud, 
   return (a.row_bits >= 64 ? 0ull : ((uint64_t)cloud << a.row_bits)) | row_idx;
 }
 
+// A lane takes a simplex.  Most simplices are settled by one or two hash probes
+// or by the first few candidates of their neighbour list (a cofacet of their own
+// diameter), so 32 of them side by side need a fraction of the instructions of a
+// warp on each; a lane that finds none among FIRST_CANDIDATES leaves the rest of
+// its list to the whole warp, 32 candidates at a time.  Bound by the L1 on dense
+// inputs that fit it and by the gathers through the rank matrix on others
+// (scattered 32-byte sectors).  D = d keeps a simplex's vertices in registers;
+// 0: any d.
+constexpr uint32_t FIRST_CANDIDATES = 32;
+
+template <int D>
 __global__ void __launch_bounds__(256) test_kernel(DimArgs a, const uint64_t* __restrict__ sidx,
                                                    const uint32_t* __restrict__ srank, uint32_t ns,
                                                    const uint8_t* __restrict__ cleared_flag /* d == 1 */,
@@ -505,114 +516,207 @@ __global__ void __launch_bounds__(256) test_kernel(DimArgs a, const uint64_t* __
                                                    uint64_t* __restrict__ col_keys, uint32_t* __restrict__ ncols,
                                                    uint32_t col_cap, unsigned long long* __restrict__ st,
                                                    int st_stride) {
-  extern __shared__ uint64_t smem[];
-  Binom B = stage_binom(a, smem);
+  const Binom B{a.binom, a.bn + 1};
   const int lane = threadIdx.x & 31;
-  const int d = a.d;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  const int d = D ? D : a.d;
+  constexpr int NV = D ? D + 1 : MAX_DIM + 2;
+  // cofacet side: (sigma, tau) zero apparent pair?  (not with the apparent-pair
+  // shortcut switched off: every simplex that is not cleared is then a column)
+  const bool apparent = !(a.opts & RIPS_OPT_NO_APPARENT);
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   // counters are flushed to the cloud's statistics whenever the warp moves to another cloud
-  unsigned long long n_cof = 0, n_fac = 0, n_clr = 0;
+  unsigned n_cof = 0, n_fac = 0, n_clr = 0;
   uint32_t cur_cloud = 0xFFFFFFFFu;
   auto flush = [&](uint32_t next) {
     if (lane == 0 && cur_cloud != 0xFFFFFFFFu) {
       unsigned long long* q = st + (size_t)cur_cloud * st_stride;
-      if (n_cof) atomicAdd(&q[4], n_cof);
-      if (n_fac) atomicAdd(&q[5], n_fac);
-      if (n_clr) atomicAdd(&q[6], n_clr);
+      if (n_cof) atomicAdd(&q[4], (unsigned long long)n_cof);
+      if (n_fac) atomicAdd(&q[5], (unsigned long long)n_fac);
+      if (n_clr) atomicAdd(&q[6], (unsigned long long)n_clr);
     }
     n_cof = n_fac = n_clr = 0;
     cur_cloud = next;
   };
-  for (uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < ns; s += warps) {
-    const uint64_t g = sidx[s];
-    if (g == ~0ull) continue;  // padding (batch plans)
-    const uint32_t r = srank[s];
-    const uint32_t cl = high_part(g, a.col_bits);
+  for (uint64_t s0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; s0 < ns; s0 += warps * 32) {
+    const uint64_t s = s0 + lane;
+    const uint64_t g = s < ns ? sidx[s] : ~0ull;
+    const bool act = g != ~0ull;  // else past the end, or padding (batch plans)
+    const unsigned am = __ballot_sync(0xffffffffu, act);
+    if (!am) continue;
+    const uint32_t cl = act ? high_part(g, a.col_bits) : 0u;
     const uint64_t idx = g & low_mask(a.col_bits);
-    if (cl != cur_cloud) flush(cl);
     // clearing: pivots of the previous dimension
-    bool cleared;
-    if (d == 1) cleared = cleared_flag[s] != 0;
-    else cleared = prev_keys != nullptr && table_find(prev_keys, prev_mask, g) >= 0;
-    if (cleared) {
-      ++n_clr;
-      continue;
+    bool clr = false, fac = false;
+    if (act) {
+      if (d == 1) clr = cleared_flag[s] != 0;
+      else clr = prev_keys != nullptr && table_find(prev_keys, prev_mask, g) >= 0;
+      // facet side (d >= 2; in dimension 1 such edges are spanning-forest edges): the previous dimension's test
+      // recorded every zero apparent pair.  A simplex is in one pair at most, so this side may go first.
+      if (!clr && apparent && d >= 2 && a.pmap) {
+        uint64_t unused;
+        fac = pair_find(a.pmap, a.pmap_mask, g, &unused);
+      }
     }
+    const bool rem = act && !clr && !fac;
     const CV cv = cloud_view(a, cl);
-    int v[MAX_DIM + 2];
-    decode(B, cv.n, idx, d, v);
-    // cofacet side: (sigma, tau) zero apparent pair?  (not with the apparent-pair
-    // shortcut switched off: every simplex that is not cleared is then a column)
-    const bool apparent = !(a.opts & RIPS_OPT_NO_APPARENT);
-    uint32_t rj[MAX_DIM + 2];
-    int hl = -1;
-    int j = apparent ? first_equal_cofacet(cv, v, d, r, lane, rj, &hl) : -1;
-    if (j >= 0) {
-      int app = 0;
-      if (lane == hl) {
-        uint32_t minus[MAX_DIM + 2];
-        ranks_minus_one(cv, v, d, minus);
-        app = 1;
-        // facets of tau dropping a vertex above j come before sigma in index order
-        for (int l = 0; l <= d && v[l] > j; ++l) {
-          uint32_t fr = minus[l];
-          for (int m2 = 0; m2 <= d; ++m2)
-            if (m2 != l) fr = max(fr, rj[m2]);
-          if (fr == r) {
-            app = 0;
+    int v[NV];
+    uint32_t rj[NV];
+    uint32_t r = 0, q = 0, end = 0;
+    int j = -1;
+    if (rem) {
+      r = srank[s];
+      int hi = cv.n - 1;
+      uint64_t N = idx;
+#pragma unroll
+      for (int l = 0; l < NV; ++l)
+        if (l <= d) {
+          const int k = d + 1 - l;
+          v[l] = k == 1 ? (int)N : max_vertex(B, k, hi, N);
+          N -= k == 1 ? N : B(v[l], k);
+          hi = v[l] - 1;
+        }
+      if (apparent) {
+        q = cv.off[v[0]];
+        end = cv.off[v[0] + 1];
+#pragma unroll
+        for (int l = 1; l < NV; ++l)
+          if (l <= d) {
+            const uint32_t o0 = cv.off[v[l]], o1 = cv.off[v[l] + 1];
+            if (o1 - o0 < end - q) {
+              q = o0;
+              end = o1;
+            }
+          }
+        const uint32_t lim = min(end, q + FIRST_CANDIDATES);
+        for (; q < lim; ++q) {
+          const int c = (int)cv.nbr[q];
+          bool ok = true;
+#pragma unroll
+          for (int l = 0; l < NV; ++l)
+            if (l <= d) {
+              rj[l] = rank_of(cv, v[l], c);
+              ok &= rj[l] <= r;  // also rejects RANK_INF and vertices of sigma
+            }
+          if (ok) {
+            j = c;
             break;
           }
         }
       }
-      app = __shfl_sync(0xffffffffu, app, hl);
-      if (app) {
-        ++n_cof;
-        if (lane == 0 && a.amap) {  // tau -> sigma, for the reduction and the next dimension
-          CofacetSums cs;
-          cofacet_sums(B, v, d, cs);
-          int c = 0;
-          for (int l = 0; l <= d; ++l) c += v[l] > j;
-          const uint64_t tidx = cs.above[c] + B(j, d + 2 - c) + cs.below[c];
-          const int64_t slot = pair_insert(a.amap, a.amap_mask, table_key(a, cl, tidx));
-          if (slot < 0) set_error(a.err, ERRF_TABLE_FULL);
-          else {
-            uint64_t ref = idx;
-            if (a.vbits) {
-              ref = 0;
-              for (int l = 0; l <= d; ++l) ref |= (uint64_t)v[l] << (l * a.vbits);
-            }
-            a.amap[2 * slot + 1] = (ref << 4) | (uint64_t)c;
+    }
+    unsigned m = __ballot_sync(0xffffffffu, rem && apparent && j < 0 && q < end);
+    while (m) {  // the rest of a lane's list, by the whole warp
+      const int L = __ffs(m) - 1;
+      m &= m - 1;
+      const CV cb = cloud_view(a, __shfl_sync(0xffffffffu, cl, L));
+      const uint32_t rb = __shfl_sync(0xffffffffu, r, L), eb = __shfl_sync(0xffffffffu, end, L);
+      int vb[NV];
+#pragma unroll
+      for (int l = 0; l < NV; ++l) vb[l] = l <= d ? __shfl_sync(0xffffffffu, v[l], L) : 0;
+      for (uint32_t q0 = __shfl_sync(0xffffffffu, q, L); q0 < eb; q0 += 32) {
+        const int c = q0 + lane < eb ? (int)cb.nbr[q0 + lane] : vb[0];  // a vertex of sigma is no candidate
+        bool ok = true;
+        uint32_t rc[NV];
+#pragma unroll
+        for (int l = 0; l < NV; ++l)
+          if (l <= d) {
+            rc[l] = rank_of(cb, vb[l], c);
+            ok &= rc[l] <= rb;
           }
+        const unsigned hit = __ballot_sync(0xffffffffu, ok);
+        if (hit) {
+          const int src = __ffs(hit) - 1;
+          const int jc = __shfl_sync(0xffffffffu, c, src);
+          if (lane == L) j = jc;
+#pragma unroll
+          for (int l = 0; l < NV; ++l)
+            if (l <= d) {
+              const uint32_t x = __shfl_sync(0xffffffffu, rc[l], src);
+              if (lane == L) rj[l] = x;
+            }
+          break;
         }
-        continue;
       }
     }
-    // facet side (d >= 2; in dimension 1 such edges are spanning-forest edges):
-    // the previous dimension's test recorded every zero apparent pair
-    if (apparent && d >= 2) {
-      bool fac;
-      if (a.pmap) {
-        uint64_t unused;
-        fac = pair_find(a.pmap, a.pmap_mask, g, &unused);
-      } else {
+    bool app = false;
+    if (j >= 0) {
+      app = true;
+      // facets of tau dropping a vertex above j come before sigma in index order: none may have its diameter
+      int c = 0;
+#pragma unroll
+      for (int l = 0; l < NV; ++l)
+        if (l <= d && v[l] > j) {
+          ++c;
+          uint32_t fr = 0;
+#pragma unroll
+          for (int x = 0; x < NV; ++x)
+            if (x <= d && x != l) {
+              fr = max(fr, rj[x]);
+#pragma unroll
+              for (int y = x + 1; y < NV; ++y)
+                if (y <= d && y != l) fr = max(fr, rank_of(cv, v[x], v[y]));
+            }
+          if (fr == r) app = false;
+        }
+      if (app && a.amap) {  // tau -> sigma, for the reduction and the next dimension
+        uint64_t tidx = B(j, d + 2 - c);
+#pragma unroll
+        for (int l = 0; l < NV; ++l)
+          if (l <= d) tidx += B(v[l], l < c ? d + 2 - l : d + 1 - l);
+        const int64_t slot = pair_insert(a.amap, a.amap_mask, table_key(a, cl, tidx));
+        if (slot < 0) {
+          set_error(a.err, ERRF_TABLE_FULL);
+        } else {
+          uint64_t ref = idx;
+          if (a.vbits) {
+            ref = 0;
+#pragma unroll
+            for (int l = 0; l < NV; ++l)
+              if (l <= d) ref |= (uint64_t)v[l] << (l * a.vbits);
+          }
+          a.amap[2 * slot + 1] = (ref << 4) | (uint64_t)c;
+        }
+      }
+    }
+    if (apparent && d >= 2 && !a.pmap) {  // no recorded pairs: a warp looks for each remaining simplex's facet
+      m = __ballot_sync(0xffffffffu, rem && !app);
+      while (m) {
+        const int L = __ffs(m) - 1;
+        m &= m - 1;
+        const CV cb = cloud_view(a, __shfl_sync(0xffffffffu, cl, L));
+        int w[MAX_DIM + 2];
+#pragma unroll
+        for (int l = 0; l < NV; ++l) w[l] = l <= d ? __shfl_sync(0xffffffffu, v[l], L) : 0;
         uint32_t minus[MAX_DIM + 2];
-        ranks_minus_one(cv, v, d, minus);
-        fac = zero_apparent_facet(cv, v, d, r, minus, lane) >= 0;
-      }
-      if (fac) {
-        ++n_fac;
-        continue;
+        ranks_minus_one(cb, w, d, minus);
+        const bool f = zero_apparent_facet(cb, w, d, __shfl_sync(0xffffffffu, r, L), minus, lane) >= 0;
+        if (lane == L) fac = f;
       }
     }
-    if (lane == 0) {
-      uint32_t pos = atomicAdd(ncols, 1u);
-      if (pos < col_cap) {
-        const int hb = a.rank_bits + a.col_bits;
-        const uint64_t key = (hb >= 64 ? 0ull : ((uint64_t)cl << hb)) |
-                             ((uint64_t)(a.rank_max - r) << a.col_bits) | idx;
-        col_keys[pos] = key;
-      } else {
-        set_error(a.err, ERRF_OUT_OVERFLOW);
+    const bool col = rem && !app && !fac;
+    const unsigned mc = __ballot_sync(0xffffffffu, app), mf = __ballot_sync(0xffffffffu, fac && !app),
+                   ml = __ballot_sync(0xffffffffu, clr), mk = __ballot_sync(0xffffffffu, col);
+    const uint32_t c0 = __shfl_sync(0xffffffffu, cl, __ffs(am) - 1);
+    if (__all_sync(0xffffffffu, !act || cl == c0)) {
+      if (c0 != cur_cloud) flush(c0);
+      n_cof += __popc(mc);
+      n_fac += __popc(mf);
+      n_clr += __popc(ml);
+    } else if (app || fac || clr) {  // clouds meet within the warp's simplices
+      atomicAdd(st + (size_t)cl * st_stride + (app ? 4 : clr ? 6 : 5), 1ull);
+    }
+    if (mk) {
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(ncols, (uint32_t)__popc(mk));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (col) {
+        const uint32_t pos = base + __popc(mk & ((1u << lane) - 1u));
+        if (pos < col_cap) {
+          const int hb = a.rank_bits + a.col_bits;
+          col_keys[pos] = (hb >= 64 ? 0ull : ((uint64_t)cl << hb)) | ((uint64_t)(a.rank_max - r) << a.col_bits) | idx;
+        } else {
+          set_error(a.err, ERRF_OUT_OVERFLOW);
+        }
       }
     }
   }
@@ -1825,11 +1929,17 @@ cudaError_t launch_test(const DimArgs& a, const uint64_t* sidx, const uint32_t* 
                         uint64_t* col_keys, uint32_t* ncols, uint32_t col_cap, unsigned long long* stats,
                         int stats_stride, cudaStream_t st) {
   if (ns == 0) return cudaSuccess;
-  size_t sm = binom_smem(a);
-  cudaError_t e = prepare(test_kernel, sm);
-  if (e != cudaSuccess) return e;
-  test_kernel<<<grid_for_warps(ns, a.scan_blocks_per_sm), 256, sm, st>>>(a, sidx, srank, ns, cleared_flag, prev_keys, prev_mask, col_keys,
-                                                   ncols, col_cap, stats, stats_stride);
+  const int grid = grid_for_warps((ns + 31) / 32, a.scan_blocks_per_sm);
+#define TEST(D) \
+  test_kernel<D><<<grid, 256, 0, st>>>(a, sidx, srank, ns, cleared_flag, prev_keys, prev_mask, col_keys, ncols, col_cap, \
+                                       stats, stats_stride)
+  switch (a.d) {
+    case 1: TEST(1); break;
+    case 2: TEST(2); break;
+    case 3: TEST(3); break;
+    default: TEST(0);
+  }
+#undef TEST
   note_launch();
   return cudaGetLastError();
 }
