@@ -1,5 +1,5 @@
 // Wide elimination: the reduction of one column by a team of blocks, many
-// additions at a time.  Included by rips_dim.cu only.
+// additions at a time.  Included by rips_reduce.cuh only.
 //
 // Algorithm 1 adds one column per pivot, and a column's next owner depends on
 // its new pivot, so a chain of additions is sequential and costs a round of
@@ -22,7 +22,7 @@
 // the rows beyond are in the table only.  A round extends the front from the mid
 // list, up to a key sampled so that about K rows join it, looks its rows over,
 // writes the live owned ones into a work list, and then adds their owners, one
-// warp a row.  The mid list is refilled by a scan of the table.  K is a third of the additions made so far (12 at
+// warp a row.  The mid list is refilled by a scan of the table.  K is a third of the additions made so far (8 at
 // first), so a chain of A additions takes on the order of log2(A) rounds and the
 // additions wasted on rows past its pivot are a share of A.  A window whose rows
 // multiply is cut back to K.  (K counts rows that have an owner: the window is
@@ -43,53 +43,6 @@
 // replicated state, separated by team barriers.  A column that outlives the
 // others is suspended between two rounds and resumed by a larger team.
 
-enum { L_FRONT = 0, L_MID = 1, L_FAR = 2 };  // L_FAR: beyond the mid list, in the table only
-
-struct WideList {
-  unsigned long long off, cap;  // arena entries [off, off + cap)
-};
-
-// what a team's threads count during one section (between two team barriers)
-struct WideCount {
-  unsigned add[2];  // rows appended to each list
-  unsigned fresh;   // rows entered into the table
-  unsigned todo;    // rows put on the work list
-  unsigned count;   // rows with an owner among those that join the front; rows of a stored run
-  unsigned nlong;   // stored runs left to the whole team
-  unsigned stop;    // 1: out of time, 2: give way to a larger team
-  unsigned long long un, ow;   // oldest live row without and with an owner
-  unsigned long long longsum;  // entries of the runs offered to the team
-  unsigned long long longroom; // and of those it takes
-  unsigned long long tmp;      // arena offset handed out by the leader
-};
-
-// Sections rotate through three sets of counters: the one in use, the one read
-// at the last barrier and the one the leader clears for the next section.
-struct WideShared {
-  WideCount c[3];
-  unsigned bar_count, bar_gen;
-};
-
-// state of a column's reduction, the same in every block of its team
-struct WideState {
-  uint32_t j, cl, step, dil;
-  int ph, tcur;
-  uint32_t n[2];
-  int cur[2];
-  WideList list[2][2];
-  WideList tab[2];
-  WideList todo, lng;
-  uint64_t tmask, used;
-  uint64_t bound, mbound;
-  unsigned long long t0;
-  WideCount d;  // the last section's counts
-};
-
-struct WideCtx {
-  WideState st;
-  WideShared sh;
-};
-
 namespace {
 
 constexpr uint32_t SORT_RUN = 1024;  // stored runs up to this length are sorted (and usable by a warp)
@@ -97,11 +50,12 @@ constexpr uint32_t SORT_RUN = 1024;  // stored runs up to this length are sorted
 // owner code of a front row: the pair map's value (low four bits: 0..8), or
 constexpr uint64_t OWN_TABLE = 13, OWN_NONE = 14, OWN_UNKNOWN = 15;  // OWN_TABLE | (ordinal << 4)
 
-constexpr uint32_t WIDE_K0 = 12;         // rows of the first window
+constexpr uint32_t WIDE_K0 = 8;         // rows of the first window
 constexpr uint32_t WIDE_SAMPLES = 128;   // keys sampled to place a bound, one a thread
 constexpr uint32_t TEAM_MIN_ROWS = 1024;  // stored rows from which a column starts with a team
 constexpr uint32_t TEAM_MIN_STEPS = 32;  // additions a block makes before it gives its column to a team
-constexpr int WIDE_MAX_BLOCKS = 1280;     // blocks of a reduction (three lists of them fit the control block)
+constexpr uint32_t TEAM_SMALL = 64;         // blocks of a lone team up to
+constexpr uint32_t TEAM_LARGE_STEPS = 4096;  // additions
 constexpr uint32_t WIDE_LONGS = 256;     // stored runs added by the whole team in one section
 
 struct Team {
@@ -673,107 +627,29 @@ __device__ int wide_refill(const Team& t, const RedState& s, WideState& w, uint3
 // ---------------------------------------------------------------- additions
 
 // The coboundary of a d-simplex (reference, rank) times f, added to the working
-// column by one warp: lanes take the neighbours of the vertex with the fewest.
-// D = d fixes the loops' lengths (vertices and sums in registers); 0: any d.
+// column by one warp.
 template <int D>
 __device__ uint32_t wide_gen(const DimArgs& a, const RedState& s, const WideState& w, const WideView& v, const CV& cv,
                              const Binom& B, int lane, uint64_t ref, bool packed, uint32_t rank, uint32_t f,
                              unsigned& fresh) {
   const int d = D ? D : a.d;
-  constexpr int NV = D ? D + 1 : MAX_DIM + 2;
-  int x[NV];
-  if (packed) {
-    const uint64_t m = (1ull << a.vbits) - 1;
-#pragma unroll
-    for (int l = 0; l < NV; ++l)
-      if (l <= d) x[l] = (int)((ref >> (l * a.vbits)) & m);
-  } else {
-    int hi = cv.n - 1;
-    uint64_t N = ref;
-#pragma unroll
-    for (int l = 0; l < NV; ++l)
-      if (l <= d) {
-        const int k = d + 1 - l;
-        x[l] = k == 1 ? (int)N : max_vertex(B, k, hi, N);
-        N -= k == 1 ? N : B(x[l], k);
-        hi = x[l] - 1;
-      }
-  }
-  // sums of the cofacet index with the new vertex below c of the simplex's vertices (CofacetSums)
-  uint64_t sum[NV + 1];
-  {
-    uint64_t acc = 0;
-#pragma unroll
-    for (int l = NV - 1; l >= 0; --l)
-      if (l <= d) acc += B(x[l], d + 1 - l);
-    sum[0] = acc;
-#pragma unroll
-    for (int l = 0; l < NV; ++l)
-      if (l <= d) sum[l + 1] = sum[l] - B(x[l], d + 1 - l) + B(x[l], d + 2 - l);
-  }
-  int best = 0;
-  uint32_t beg = cv.off[x[0]], end = cv.off[x[0] + 1];
-#pragma unroll
-  for (int l = 1; l < NV; ++l)
-    if (l <= d) {
-      const uint32_t o0 = cv.off[x[l]], o1 = cv.off[x[l] + 1];
-      if (o1 - o0 < end - beg) {
-        best = l;
-        beg = o0;
-        end = o1;
-      }
-    }
+  Coboundary<D> cob;
+  cob.set(a, cv, B, ref, packed);
   uint32_t cnt = 0;
-  constexpr int U = 4;  // candidates a lane under way together: a coboundary is a few dependent memory round trips
-  for (uint32_t q0 = beg; q0 < end; q0 += 32 * U) {
-    bool ok[U];
-    int j[U], c[U];
-    uint32_t r[U], f4[U];
-    uint64_t key[U];
+  for (uint32_t q0 = cob.beg; q0 < cob.end; q0 += 32 * Coboundary<D>::U) {
+    bool ok[Coboundary<D>::U];
+    uint64_t key[Coboundary<D>::U];
+    int c[Coboundary<D>::U];
+    uint32_t f4[Coboundary<D>::U];
+    cob.eval(a, cv, B, rank, q0, lane, ok, key, c);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint32_t q = q0 + u * 32 + lane;
-      ok[u] = q < end;
-      j[u] = ok[u] ? (int)cv.nbr[q] : x[0];  // a vertex of the simplex is no candidate
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      r[u] = rank;
-      c[u] = 0;
-#pragma unroll
-      for (int l = 0; l < NV; ++l)
-        if (l <= d) {
-          const uint32_t q = q0 + u * 32 + lane;
-          const uint32_t y = cv.nrank && l == best && q < end ? cv.nrank[q] : rank_of(cv, x[l], j[u]);
-          ok[u] &= y != RANK_INF;
-          r[u] = max(r[u], y);
-          c[u] += x[l] > j[u];
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      uint64_t si = sum[0];
-#pragma unroll
-      for (int l = 1; l <= NV; ++l)
-        if (l <= d + 1) si = c[u] == l ? sum[l] : si;
-      key[u] = row_key(a, r[u], si + B(j[u], d + 2 - c[u]));
+    for (int u = 0; u < Coboundary<D>::U; ++u) {
       f4[u] = a.p == 2 ? 1u : (((d - c[u]) & 1) ? a.p - f : f);
       cnt += __popc(__ballot_sync(0xffffffffu, ok[u]));
     }
     fresh += wide_insert(s, w, v, lane, a.p, ok, key, f4);
   }
   return cnt;
-}
-
-__device__ uint32_t wide_gen_any(const DimArgs& a, const RedState& s, const WideState& w, const WideView& v,
-                                 const CV& cv, const Binom& B, int lane, uint64_t ref, bool packed, uint32_t rank,
-                                 uint32_t f, unsigned& fresh) {
-  switch (a.d) {
-    case 1: return wide_gen<1>(a, s, w, v, cv, B, lane, ref, packed, rank, f, fresh);
-    case 2: return wide_gen<2>(a, s, w, v, cv, B, lane, ref, packed, rank, f, fresh);
-    case 3: return wide_gen<3>(a, s, w, v, cv, B, lane, ref, packed, rank, f, fresh);
-    default: return wide_gen<0>(a, s, w, v, cv, B, lane, ref, packed, rank, f, fresh);
-  }
 }
 
 // a stored run times f, added by the `warps` warps of which this is the i-th
@@ -1009,6 +885,7 @@ __device__ __forceinline__ void wide_check(const DimArgs& a, const RedState& s, 
 }
 
 // Second section: work records [p0, p1), a warp each.
+template <int D>
 __device__ void wide_process(const DimArgs& a, const RedState& s, const Team& t, const WideState& w, const CV& cv,
                              const Binom& B, uint32_t p0, uint32_t p1) {
   const int lane = threadIdx.x & 31;
@@ -1025,7 +902,7 @@ __device__ void wide_process(const DimArgs& a, const RedState& s, const Team& t,
       wide_run(s, w, v, lane, a.p, ref, len, f, 0, 1, fresh);
       ents += len;
     } else {
-      ents += wide_gen_any(a, s, w, v, cv, B, lane, ref, kind == REC_PACKED, rank, f, fresh);
+      ents += wide_gen<D>(a, s, w, v, cv, B, lane, ref, kind == REC_PACKED, rank, f, fresh);
     }
   }
   wide_count_fresh(v.c, lane, fresh);
@@ -1057,6 +934,7 @@ __device__ void wide_longs(const RedState& s, const Team& t, const WideState& w,
 // ---------------------------------------------------------------- a column
 
 // Column j's own entries into an empty working column.
+template <int D>
 __device__ __forceinline__ int wide_begin(const DimArgs& a, const RedState& s, const Team& t, WideState& w, const CV& cv,
                           const Binom& B, uint32_t j, uint32_t cl, uint64_t jidx, uint32_t jrank) {
   const int lane = threadIdx.x & 31;
@@ -1105,7 +983,7 @@ __device__ __forceinline__ int wide_begin(const DimArgs& a, const RedState& s, c
   const uint32_t tw = (uint32_t)t.rank * WARPS_PER_BLOCK + (threadIdx.x >> 5);
   unsigned fresh = 0;
   if (jn) wide_run(s, w, v, lane, a.p, s.r_off[j], jn, 1, tw, (uint32_t)t.size * WARPS_PER_BLOCK, fresh);
-  else if (tw == 0) wide_gen_any(a, s, w, v, cv, B, lane, jidx, false, jrank, 1, fresh);
+  else if (tw == 0) wide_gen<D>(a, s, w, v, cv, B, lane, jidx, false, jrank, 1, fresh);
   wide_count_fresh(v.c, lane, fresh);
   return wide_sync(t, s, w) ? CH_DONE : CH_LONG;
 }
@@ -1125,6 +1003,7 @@ struct GiveWay {
 // Eliminates until the pivot is free, owned by a later column, or the column is
 // zero: CH_DONE with the pivot (IDX_NONE: zero) and its coefficient.  CH_HEAVY:
 // suspended between two rounds, to be resumed by a larger team.
+template <int D>
 __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s, const Team& t, WideState& w, const CV& cv,
                                             const Binom& B, uint64_t* sm, uint64_t* piv, uint32_t* coef,
                                             const GiveWay& give_way) {
@@ -1227,7 +1106,7 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
           (uint32_t)min((unsigned long long)(todo - p0), max(64ull, ((unsigned long long)w.used + 65536) >> sbits));
       const int e = wide_ensure(t, s, w, p, (unsigned long long)most << sbits);
       if (e != CH_DONE) return e;
-      wide_process(a, s, t, w, cv, B, p0, p0 + most);
+      wide_process<D>(a, s, t, w, cv, B, p0, p0 + most);
       if (!wide_sync(t, s, w)) return CH_LONG;
       grown += w.d.add[L_FRONT];
       p0 += most;
