@@ -243,7 +243,7 @@ RIPS_API int rips_barcodes_backward_dist(const rips_result_t* res, const float* 
  * callers that cannot allocate device memory while they run (a serving process
  * whose memory pool already owns the whole device, a real-time loop that must
  * not wait on cudaMalloc / cudaFree, which may synchronise the device).  All
- * intermediate data lives in a fixed file-scope device array (about 3.3 MB,
+ * intermediate data lives in a fixed file-scope device array (about 2.3 MB,
  * held by every GPU that loads the library until the process exits), so n is
  * at most RIPS_NOALLOC_MAX_N; larger n returns RIPS_ERR_BAD_ARG.
  * d_dist: n x n FP32 (DEVICE, strict lower triangle read, as for

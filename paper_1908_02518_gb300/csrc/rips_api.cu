@@ -510,8 +510,6 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
 
   // ---------------- H0
   CR(grow_keep(w.bars, ((size_t)N + 16) * sizeof(rips_bar_t), 0, s));
-  CR(ensure(w.eu, (size_t)(m + 1) * 4));
-  CR(ensure(w.ev, (size_t)(m + 1) * 4));
   CR(ensure(w.inforest, (size_t)m + 1));
   CR(ensure(w.nbars, 16));
   CR(ensure(w.stats, (size_t)C * SPC * 8));
@@ -521,12 +519,13 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
   {
     KTimer kt(w, RIPS_K_H0, s);
     if (h0_blocks_fit(n_max)) {
-      CK(launch_h0_blocks(dclouds, C, n_max, keys, eb, P<uint32_t>(w.eu), P<uint32_t>(w.ev), m,
-                          P<uint8_t>(w.inforest), P<rips_bar_t>(w.bars), P<uint32_t>(w.nbars),
-                          (uint32_t)(w.bars.cap / sizeof(rips_bar_t)), dstats, SPC, P<uint32_t>(w.err), s));
+      CK(launch_h0_blocks(dclouds, C, n_max, keys, eb, m, P<uint8_t>(w.inforest), P<rips_bar_t>(w.bars),
+                          P<uint32_t>(w.nbars), (uint32_t)(w.bars.cap / sizeof(rips_bar_t)), dstats, SPC, s));
     } else {
       if (C != 1) return RIPS_ERR_BAD_ARG;
       const int n = n_max;
+      CR(ensure(w.eu, (size_t)(m + 1) * 4));
+      CR(ensure(w.ev, (size_t)(m + 1) * 4));
       CR(ensure(w.comp, (size_t)n * 4));
       CR(ensure(w.best, (size_t)n * 4));
       CR(ensure(w.parent, (size_t)n * 4));
@@ -1233,8 +1232,6 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   CR(ensure(w.binom, (size_t)(kmax + 1) * (pl.n_max + 1) * 8));
   CR(ensure(w.cdist, pl.RR * 4));
   CR(ensure(w.bars, (N + E + 16) * sizeof(rips_bar_t)));
-  CR(ensure(w.eu, (E + 1) * 4));
-  CR(ensure(w.ev, (E + 1) * 4));
   CR(ensure(w.inforest, E + 1));
   CR(ensure(w.nbars, 16));
   CR(ensure(w.stats, SPCB));
@@ -1326,9 +1323,8 @@ int plan_run(PlanState& pl, const float* d_points, cudaStream_t s) {
   CK(launch_binomial_table(P<uint64_t>(w.binom), pl.n_max, 3, s));
   // H0, one block per cloud (edges at the cloud table's offsets, set on the device)
   const uint32_t bar_cap = (uint32_t)(w.bars.cap / sizeof(rips_bar_t));
-  CK(launch_h0_blocks(dclouds, C, pl.n_max, keys, pl.eb, P<uint32_t>(w.eu), P<uint32_t>(w.ev), (uint32_t)E,
-                      P<uint8_t>(w.inforest), P<rips_bar_t>(w.bars), P<uint32_t>(w.nbars), bar_cap, dstats, PLAN_SPC,
-                      P<uint32_t>(w.err), s));
+  CK(launch_h0_blocks(dclouds, C, pl.n_max, keys, pl.eb, (uint32_t)E, P<uint8_t>(w.inforest), P<rips_bar_t>(w.bars),
+                      P<uint32_t>(w.nbars), bar_cap, dstats, PLAN_SPC, s));
   // dimension 1 over all E slots (the padding is skipped)
   const DimArgs& a = pl.a;
   unsigned long long* st = dstats + 16;

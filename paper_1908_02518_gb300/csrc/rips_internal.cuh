@@ -255,9 +255,8 @@ struct RedState {
 // per-cloud H0 in one block per cloud (every n_c small enough for shared memory)
 bool h0_blocks_fit(int n_max);
 cudaError_t launch_h0_blocks(const CloudInfo* clouds, int nclouds, int n_max, const uint64_t* sorted_keys,
-                             int edge_bits, uint32_t* eu, uint32_t* ev, uint32_t m_total, uint8_t* in_forest,
-                             rips_bar_t* bars, uint32_t* nbars, uint32_t bar_cap, unsigned long long* stats,
-                             int stats_stride, uint32_t* err, cudaStream_t s);
+                             int edge_bits, uint32_t m_total, uint8_t* in_forest, rips_bar_t* bars, uint32_t* nbars,
+                             uint32_t bar_cap, unsigned long long* stats, int stats_stride, cudaStream_t s);
 // one large cloud: Boruvka rounds over the whole GPU, then the elder rule
 cudaError_t run_h0_large(int n, const uint64_t* sorted_keys, uint32_t m, int edge_bits, uint32_t* eu, uint32_t* ev,
                          uint32_t* comp, uint32_t* best, uint32_t* parent, uint8_t* in_forest, uint32_t* flags,

@@ -8,7 +8,7 @@
 // time).  For them, rips_h0_barcode_noalloc computes the dimension-0 barcode
 // of one distance matrix of at most RIPS_NOALLOC_MAX_N points without any
 // allocation: every intermediate buffer lives in one file-scope device array
-// of fixed size (NOALLOC_BYTES below, about 3.3 MB), which every GPU that
+// of fixed size (NOALLOC_BYTES below, about 2.3 MB), which every GPU that
 // loads the library holds until the process exits.  The caller passes the
 // matrix and the output buffers.
 //
@@ -39,9 +39,7 @@ static_assert(NA_MAX_EDGES < (1ull << NA_EDGE_BITS), "edge index bits");
 constexpr size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t OFF_KEYS = 0;
 constexpr size_t OFF_KEYS_ALT = OFF_KEYS + al(NA_MAX_EDGES * 8);
-constexpr size_t OFF_EU = OFF_KEYS_ALT + al(NA_MAX_EDGES * 8);
-constexpr size_t OFF_EV = OFF_EU + al(NA_MAX_EDGES * 4);
-constexpr size_t OFF_FOREST = OFF_EV + al(NA_MAX_EDGES * 4);
+constexpr size_t OFF_FOREST = OFF_KEYS_ALT + al(NA_MAX_EDGES * 8);
 constexpr size_t OFF_ROWMAX = OFF_FOREST + al(NA_MAX_EDGES);
 constexpr size_t OFF_VCLOUD = OFF_ROWMAX + al(NA_MAX_N * 4);
 constexpr size_t OFF_CLOUD = OFF_VCLOUD + al(NA_MAX_N * 4);
@@ -123,8 +121,6 @@ extern "C" RIPS_API int rips_h0_barcode_noalloc(const float* d_dist, int64_t n, 
   cudaStream_t s = (cudaStream_t)cuda_stream;
   uint64_t* keys = (uint64_t*)(base + OFF_KEYS);
   uint64_t* keys_alt = (uint64_t*)(base + OFF_KEYS_ALT);
-  uint32_t* eu = (uint32_t*)(base + OFF_EU);
-  uint32_t* ev = (uint32_t*)(base + OFF_EV);
   uint8_t* forest = base + OFF_FOREST;
   uint32_t* rowmax = (uint32_t*)(base + OFF_ROWMAX);
   uint32_t* vcloud = (uint32_t*)(base + OFF_VCLOUD);
@@ -168,8 +164,8 @@ extern "C" RIPS_API int rips_h0_barcode_noalloc(const float* d_dist, int64_t n, 
     e = cudaGetLastError();
   }
   if (e == cudaSuccess)
-    e = launch_h0_blocks(cloud, 1, (int)n, sorted, NA_EDGE_BITS, eu, ev, (uint32_t)m_cap, forest, d_bars, d_nbars,
-                         (uint32_t)n, stats, 16, counts + 1, s);
+    e = launch_h0_blocks(cloud, 1, (int)n, sorted, NA_EDGE_BITS, (uint32_t)m_cap, forest, d_bars, d_nbars, (uint32_t)n,
+                         stats, 16, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return RIPS_ERR_CUDA;
