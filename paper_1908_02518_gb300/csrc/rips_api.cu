@@ -949,27 +949,28 @@ int batched_locked(Workspace& w, const float* d_points, const int64_t* offsets, 
   r->k = k;
   std::vector<int64_t> ns(batch);
   std::vector<CloudInfo> ci(batch);
-  std::vector<uint32_t> row_off(batch + 1, 0);
-  uint64_t RR = 0, rows = 0;
+  std::vector<uint32_t> tile_off(batch + 1, 0);
+  uint64_t RR = 0, tiles = 0;
   int64_t nmax = 1;
   for (int32_t c = 0; c < batch; ++c) {
     ns[c] = offsets[c + 1] - offsets[c];
     nmax = std::max<int64_t>(nmax, ns[c]);
     ci[c] = CloudInfo{(int)ns[c], (uint32_t)offsets[c], RR, 0, 0, 0.0f, 0};
     RR += (uint64_t)ns[c] * ns[c];
-    row_off[c] = (uint32_t)rows;
-    rows += (ns[c] + 7) / 8;
+    tile_off[c] = (uint32_t)tiles;
+    const uint64_t nb = ((uint64_t)ns[c] + 31) / 32;
+    tiles += nb * (nb + 1) / 2;
   }
-  row_off[batch] = (uint32_t)rows;
-  int rc = ensure(w.cdist, RR * 4);
+  tile_off[batch] = (uint32_t)tiles;
+  int rc = tiles > 0x7FFFFFFFull ? RIPS_ERR_OVERFLOW : ensure(w.cdist, RR * 4);
   if (rc == RIPS_OK) rc = ensure(w.clouds, (size_t)batch * sizeof(CloudInfo));
   if (rc == RIPS_OK) rc = ensure(w.tileoff, (size_t)(batch + 1) * 4);
   if (rc == RIPS_OK) {
     if (cudaMemcpyAsync(w.clouds.p, ci.data(), (size_t)batch * sizeof(CloudInfo), cudaMemcpyHostToDevice, s) !=
             cudaSuccess ||
-        cudaMemcpyAsync(w.tileoff.p, row_off.data(), (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, s) !=
+        cudaMemcpyAsync(w.tileoff.p, tile_off.data(), (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, s) !=
             cudaSuccess ||
-        launch_distance_matrices(d_points, k, P<CloudInfo>(w.clouds), P<uint32_t>(w.tileoff), batch, (uint32_t)rows,
+        launch_distance_matrices(d_points, k, P<CloudInfo>(w.clouds), P<uint32_t>(w.tileoff), batch, (uint32_t)tiles,
                                  P<float>(w.cdist), s) != cudaSuccess) {
       cudaGetLastError();
       rc = RIPS_ERR_CUDA;
@@ -1101,7 +1102,7 @@ struct PlanState {
   uint32_t p = 2;
   int n_max = 1;
   std::vector<int64_t> ns, offsets;
-  uint64_t N = 0, RR = 0, e_cap = 0, drows = 0, vtiles = 0;
+  uint64_t N = 0, RR = 0, e_cap = 0, vtiles = 0;
   int eb = 0, cb = 0;
   DimArgs a{};
   uint32_t tcap = 0;
@@ -1109,7 +1110,7 @@ struct PlanState {
   size_t arena = 0;
   int blocks = 0;
   uint32_t slice = 0;
-  Buf clouds0, dtile;
+  Buf clouds0;
 };
 
 constexpr int PLAN_SPC = 32;  // statistics counters per cloud (dimensions 0 and 1)
@@ -1129,8 +1130,7 @@ void release_plan(PlanState& pl) {
                 &w.r_len, &w.reduced, &w.claim, &w.reduce, &w.heavy, &w.lists, &w.r_key, &w.r_coef, &w.r_top, &w.wide,
                 &w.tkeys[0], &w.tkeys[1], &w.tvals[0], &w.tvals[1], &w.amk[0], &w.amk[1],
                 &w.bars, &w.bars_alt, &w.bk0, &w.bk1, &w.bp0, &w.bp1, &w.bartmp, &w.nbars, &w.stats,
-                &w.bwd_bars, &w.bwd_off, &w.cdist, &w.clouds, &w.tileoff, &w.vcloud, &w.ccounts, &pl.clouds0,
-                &pl.dtile};
+                &w.bwd_bars, &w.bwd_off, &w.cdist, &w.clouds, &w.tileoff, &w.vcloud, &w.ccounts, &pl.clouds0};
   for (Buf* b : all) release(*b);
 }
 
@@ -1146,26 +1146,23 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   pl.offsets.assign(offsets, offsets + batch + 1);
   pl.ns.resize(batch);
   std::vector<CloudInfo> ci(batch);
-  std::vector<uint32_t> dtile(batch + 1), vtile(batch + 1);
+  std::vector<uint32_t> vtile(batch + 1);
   for (int32_t c = 0; c < batch; ++c) {
     const int64_t n = offsets[c + 1] - offsets[c];
     if (n < 1 || n > 46340) return RIPS_ERR_BAD_ARG;
     pl.ns[c] = n;
     pl.n_max = std::max<int>(pl.n_max, (int)n);
     ci[c] = CloudInfo{(int)n, (uint32_t)(offsets[c] - offsets[0]), pl.RR, 0, 0, 0.0f, 0};
-    dtile[c] = (uint32_t)pl.drows;
     vtile[c] = (uint32_t)pl.vtiles;
     const uint64_t nb = ((uint64_t)n + 31) / 32;
     pl.N += (uint64_t)n;
     pl.RR += (uint64_t)n * (uint64_t)n;
     pl.e_cap += (uint64_t)n * (uint64_t)(n - 1) / 2;
-    pl.drows += ((uint64_t)n + 7) / 8;
     pl.vtiles += nb * (nb + 1) / 2;
   }
-  dtile[batch] = (uint32_t)pl.drows;
   vtile[batch] = (uint32_t)pl.vtiles;
   if (pl.e_cap == 0 || !h0_blocks_fit(pl.n_max)) return RIPS_ERR_BAD_ARG;
-  if (pl.N > 0xFFFFFFF0ull || pl.e_cap > 0x7FFFFFF0ull || pl.vtiles > 0x7FFFFFFFull || pl.drows > 0x7FFFFFFFull)
+  if (pl.N > 0xFFFFFFF0ull || pl.e_cap > 0x7FFFFFF0ull || pl.vtiles > 0x7FFFFFFFull)
     return RIPS_ERR_OVERFLOW;
   pl.cb = batch > 1 ? bit_width64((uint64_t)batch - 1) : 0;
   pl.eb = bits_of_count(host_binom((uint64_t)pl.n_max, 2));
@@ -1213,7 +1210,6 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   const size_t SPCB = (size_t)batch * PLAN_SPC * 8;
   CR(ensure(w.clouds, (size_t)batch * sizeof(CloudInfo)));
   CR(ensure(pl.clouds0, (size_t)batch * sizeof(CloudInfo)));
-  CR(ensure(pl.dtile, (size_t)(batch + 1) * 4));
   CR(ensure(w.tileoff, (size_t)(batch + 1) * 4));
   CR(ensure(w.vcloud, N * 4));
   CR(ensure(w.ccounts, (size_t)(batch + 1) * 4));
@@ -1257,7 +1253,6 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   CR(ensure(w.r_coef, pl.arena * 4));
   w.r_cap = pl.arena;
   if (cudaMemcpy(pl.clouds0.p, ci.data(), (size_t)batch * sizeof(CloudInfo), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(pl.dtile.p, dtile.data(), (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(w.tileoff.p, vtile.data(), (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaGetLastError();
     return RIPS_ERR_CUDA;
@@ -1294,7 +1289,7 @@ int plan_run(PlanState& pl, const float* d_points, cudaStream_t s) {
   CK(cudaMemsetAsync(w.ccounts.p, 0, (size_t)(C + 1) * 4, s));
   CK(cudaMemsetAsync(w.stats.p, 0, (size_t)C * PLAN_SPC * 8, s));
   CK(cudaMemsetAsync(w.nbars.p, 0, 16, s));
-  CK(launch_distance_matrices(pts, pl.k, dclouds, P<uint32_t>(pl.dtile), C, (uint32_t)pl.drows, P<float>(w.cdist), s));
+  CK(launch_distance_matrices(pts, pl.k, dclouds, P<uint32_t>(w.tileoff), C, (uint32_t)pl.vtiles, P<float>(w.cdist), s));
   const float* dD = P<float>(w.cdist);
   // prologue
   CK(launch_cloud_vertices(dclouds, C, P<uint32_t>(w.vcloud), s));

@@ -21,7 +21,7 @@ namespace {
 constexpr int H0_BLOCK_MAX_N = 12800;  // 12 bytes of shared memory per vertex, beside the edge list
 
 __device__ __forceinline__ void edge_vertices_u32(uint64_t idx, uint32_t* a, uint32_t* b) {
-  uint32_t x = (uint32_t)((1.0 + sqrt(1.0 + 8.0 * (double)idx)) * 0.5);
+  uint32_t x = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)idx)) * 0.5f);
   while ((uint64_t)x * (x - 1) / 2 > idx) --x;
   while ((uint64_t)(x + 1) * x / 2 <= idx) ++x;
   *a = x;
