@@ -941,8 +941,8 @@ __device__ bool grid_barrier(unsigned* count, unsigned* gen, const RedState& s, 
 // round's claims are reduced in its reduce phase: heavy columns (flagged when a
 // warp gave them up) one block each, the others one warp each, both handed out
 // by atomic counters; when there are no more columns than blocks, every column
-// gets a block, and when there are no more than a quarter as many and one is
-// large, a team of blocks.  Once three blocks of four have nothing left to do, the columns
+// gets a block, and when there are no more than half as many and one is large, a
+// team of blocks.  Once half of the blocks have nothing left to do, the columns
 // still running are suspended and each goes on with a team of as many blocks as
 // the grid has for it, in as many steps as it takes (wide_advance).  Work-list
 // counters are double buffered by round parity (ctl[0..1] claim, ctl[2..3]
@@ -984,10 +984,10 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
   uint32_t* heavy[2] = {s.heavy_list, s.heavy_list + (size_t)s.ncols + 1};
   const uint32_t ncols = s.ncols_dev ? *s.ncols_dev : s.ncols;
 
-  // additions a warp makes on a column in this phase: none when blocks can take them all
-  // (unless its coboundaries fit the warp's tile: a warp then makes the first few as fast)
-  const uint32_t first_limit =
-      ncols <= BLOCK_COLUMNS * gridDim.x && s.scr_slice > SORT_TILE ? 0u : min(a.chain_limit, FIRST_CHAIN);
+  // Additions a warp makes on a column in this phase: a few while its coboundaries fit the warp's tile, else none
+  // (sorting them in the arena takes a warp longer than a block needs for the column).
+  const bool tiles = s.scr_slice <= SORT_TILE;
+  const uint32_t first_limit = tiles ? min(a.chain_limit, FIRST_CHAIN) : 0u;
   for (uint32_t j = warp_id; j < ncols; j += warps)
     init_column<D>(a, s, B, lane, tile, j, first_limit, &claim_cnt[0], &heavy_cnt[0], heavy[0]);
   if (!grid_barrier(bar_count, bar_gen, s, a.err)) return;
@@ -1018,12 +1018,12 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
     }
     const uint32_t nred = *(volatile unsigned*)&red_cnt[src];
     const uint32_t nheavy = *(volatile unsigned*)&heavy_cnt[src];
-    const bool few = nred + nheavy <= BLOCK_COLUMNS * gridDim.x;  // blocks take all columns, a few each
+    const bool few = !tiles || nred + nheavy <= BLOCK_COLUMNS * gridDim.x;  // blocks take all columns, a few each
     const uint32_t nwide = few ? nred + nheavy : nheavy;
     const uint32_t nlight = few ? 0u : nred;
-    // no more than one column for four blocks, and one of them stored with so many rows that it takes a block long to
+    // no more than one column for two blocks, and one of them stored with so many rows that it takes a block long to
     // enter them: a team each from the start
-    bool direct = nlight == 0 && 4 * nwide <= gridDim.x;
+    bool direct = nlight == 0 && 2 * nwide <= gridDim.x;
     if (direct) {
       const uint32_t j = threadIdx.x < nheavy ? heavy[src][threadIdx.x]
                          : threadIdx.x < nwide ? s.reduce_list[threadIdx.x - nheavy] : 0u;
@@ -1065,7 +1065,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
       WideCtx* c = s.wide + blockIdx.x;
       WideState& w = queue ? ws : wt;
       Team team{1, 0, &wsh};
-      GiveWay gw{heavy_next, light_next, bar_count, nwide, nlight, 3 * gridDim.x, TEAM_MIN_STEPS};
+      GiveWay gw{heavy_next, light_next, bar_count, nwide, nlight, gridDim.x, TEAM_MIN_STEPS};
       if (queue) {
         j = qt < nheavy ? heavy[src][qt] : s.reduce_list[qt - nheavy];
         if (threadIdx.x == 0) ws.tmask = 0;  // not begun
@@ -1091,7 +1091,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
         }
         const volatile unsigned* done = team_done + it % 3;
         gw = small ? GiveWay{done, done, done, 0u, 0u, 0u, TEAM_LARGE_STEPS}
-                   : GiveWay{done, done, done, nteam > 1 ? 0u : ~0u, 0u, 3 * nteam, 0u};
+                   : GiveWay{done, done, done, nteam > 1 ? 0u : ~0u, 0u, nteam, 0u};
       }
       __syncthreads();
       if (team.size) {

@@ -399,8 +399,8 @@ __device__ __forceinline__ bool wide_live(uint32_t v, uint32_t p) { return p == 
 
 // Room for `room` more rows: in both lists, and in the table at half load.  A
 // table too full is rebuilt from the rows of the front and the live rows beyond
-// it (the mid list drops its dead rows with the table), twice if that shows more
-// of them alive than there is room for.
+// it (the mid list drops its dead rows with the table), at a size for as many of
+// them as a sample of its slots shows, and again if there are more.
 __device__ int wide_ensure(const Team& t, const RedState& s, WideState& w, uint32_t p, unsigned long long room) {
   const int lane = threadIdx.x & 31;
   for (int l = 0; l < 2; ++l)
@@ -408,7 +408,19 @@ __device__ int wide_ensure(const Team& t, const RedState& s, WideState& w, uint3
   // (the second time unless a quarter of that is left free, or the next section would be back here)
   bool rebuilt = false;
   while (2 * (w.used + room) > (rebuilt ? (w.tmask + 1) / 4 * 3 : w.tmask + 1)) {
-    const unsigned long long cap = wide_pow2(rebuilt ? 4 * (w.used + room) : w.used + 2 * room);
+    unsigned long long need = 4 * (w.used + room);
+    if (!rebuilt) {  // live rows among WIDE_SAMPLES slots (every block takes the same ones)
+      bool live = false;
+      if (threadIdx.x < WIDE_SAMPLES) {
+        const unsigned long long at = w.tab[w.tcur].off + threadIdx.x * ((w.tmask + 1) / WIDE_SAMPLES);
+        const uint64_t key = __ldcg(s.r_key + at);
+        live = key != IDX_NONE && key > w.bound && wide_live(__ldcg(s.r_coef + at), p);
+      }
+      const unsigned long long seen = (unsigned)__syncthreads_count(live) + 4;
+      const unsigned long long kept = min((unsigned long long)w.used, seen * ((w.tmask + 1) / WIDE_SAMPLES) + w.n[L_FRONT]);
+      need = max(w.used + room, 3 * (kept + room));  // never less than what could be kept
+    }
+    const unsigned long long cap = wide_pow2(need);
     if (cap > (1ull << 32)) return CH_ARENA;
     if (!wide_table(t, s, w, cap)) return CH_ARENA;
     if (!wide_alt(t, s, w, L_MID, w.n[L_MID] + room)) return CH_ARENA;
@@ -990,13 +1002,13 @@ __device__ __forceinline__ int wide_begin(const DimArgs& a, const RedState& s, c
 
 // When a column gives way to a larger team (asked by its leader between rounds):
 // a block once it has made TEAM_MIN_STEPS additions, all columns and light ones
-// are handed out and three blocks of four wait; a team once three teams of four
-// are done.
+// are handed out and half of the blocks wait; a team once half of the teams are
+// done.
 struct GiveWay {
   const volatile unsigned *a, *b, *c;
   unsigned na, nb, nc, steps;
   __device__ __forceinline__ bool operator()(uint32_t step) const {
-    return step >= steps && *a >= na && *b >= nb && 4 * *c >= nc;
+    return step >= steps && *a >= na && *b >= nb && 2 * *c >= nc;
   }
 };
 
@@ -1008,7 +1020,7 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
                                             const Binom& B, uint64_t* sm, uint64_t* piv, uint32_t* coef,
                                             const GiveWay& give_way) {
   const uint32_t p = a.p;
-  const uint32_t kmax = 4u * (uint32_t)t.size * WARPS_PER_BLOCK;  // more than this and a round's time is its additions'
+  const uint32_t kmax = 2u * (uint32_t)t.size * WARPS_PER_BLOCK;  // more than this and a round's time is its additions'
   const unsigned long long rows = 1024ull * t.size * WARPS_PER_BLOCK;  // most rows a window is extended by
   const int sbits = 31 - __clz(s.scr_slice);                           // scr_slice is a power of two
   float again = 0.0f;       // share of a round's rows that come back live in the next one
