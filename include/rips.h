@@ -285,6 +285,11 @@ RIPS_API float rips_result_threshold(const rips_result_t* res, int32_t cloud);
 RIPS_API int rips_result_stats(const rips_result_t* res, int32_t cloud, int32_t dim,
                                rips_stats_t* out);
 
+/* Statistics of every cloud and dimension and the effective threshold of every
+ * cloud in one call: stats receives clouds x (dim_max + 1) entries, cloud by
+ * cloud, thresholds one per cloud; either may be NULL. */
+RIPS_API int rips_result_all_stats(const rips_result_t* res, rips_stats_t* stats, float* thresholds);
+
 /* Device-side timing of the last call's phases in milliseconds (CUDA events on
  * the call's stream), for profiling: index 0 = prologue + H_0, then one entry
  * per dimension 1..dim_max.  Returns the number of entries written. */

@@ -30,6 +30,9 @@ BAR_DTYPE = np.dtype({
     "offsets": [0, 4, 8, 12, 16, 24], "itemsize": 32})
 
 
+_STATS = tuple(f for f, _ in _lib.Stats._fields_)  # all 64-bit counters
+
+
 @dataclass
 class Result:
     """Bars and statistics of one call (copied out of the library's result)."""
@@ -81,14 +84,11 @@ def _collect(lib, handle, keep_handle: bool) -> Result:
         C.memmove(arr.ctypes.data, ptr, nb * 32)
     clouds = lib.rips_result_num_clouds(handle)
     dim_max = lib.rips_result_dim_max(handle)
-    stats = []
-    for c in range(clouds):
-        row = []
-        for d in range(dim_max + 1):
-            s = _lib.Stats()
-            lib.rips_result_stats(handle, c, d, C.byref(s))
-            row.append({f: int(getattr(s, f)) for f, _ in _lib.Stats._fields_})
-        stats.append(row)
+    flat = np.empty((clouds, dim_max + 1, len(_STATS)), dtype=np.int64)
+    thresholds = np.empty(clouds, dtype=np.float32)
+    _lib.check(lib.rips_result_all_stats(handle, flat.ctypes.data_as(C.POINTER(_lib.Stats)),
+                                         thresholds.ctypes.data_as(C.POINTER(C.c_float))), "rips_result_all_stats")
+    stats = [[dict(zip(_STATS, s)) for s in row] for row in flat.tolist()]
     ph = (C.c_float * 16)()
     k = lib.rips_result_phase_ms(handle, ph, 16)
     kms = {}
@@ -97,7 +97,7 @@ def _collect(lib, handle, keep_handle: bool) -> Result:
         reg = C.c_int64()
         lib.rips_result_kernel_ms(handle, q, C.byref(ms), C.byref(reg))
         kms[name] = (float(ms.value), int(reg.value))
-    res = Result(arr, [float(lib.rips_result_threshold(handle, c)) for c in range(clouds)], stats,
+    res = Result(arr, thresholds.tolist(), stats,
                  [float(ph[i]) for i in range(max(k, 0))], kms, dim_max, clouds)
     if keep_handle:
         res._handle = handle

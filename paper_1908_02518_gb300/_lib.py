@@ -43,7 +43,7 @@ class Tuning(C.Structure):
 EXPORTS = [
     "rips_barcodes", "rips_barcodes_device", "rips_distance_matrix_device", "rips_barcodes_batched",
     "rips_barcodes_backward", "rips_barcodes_packed", "rips_barcodes_sparse", "rips_barcodes_sparse_points", "rips_barcodes_batched_dists", "rips_barcodes_backward_dist", "rips_result_num_bars", "rips_result_bars", "rips_result_num_clouds",
-    "rips_result_dim_max", "rips_result_threshold", "rips_result_stats", "rips_result_phase_ms",
+    "rips_result_dim_max", "rips_result_threshold", "rips_result_stats", "rips_result_all_stats", "rips_result_phase_ms",
     "rips_result_free", "rips_status_string", "rips_kernel_launch_count", "rips_set_kernel_timing",
     "rips_result_kernel_ms", "rips_h0_barcode_noalloc", "rips_set_tuning", "rips_get_tuning", "rips_clear_tuning",
     "rips_set_limits", "rips_get_limits", "rips_set_options", "rips_get_options", "rips_batch_plan_create", "rips_batch_plan_run", "rips_batch_plan_result",
@@ -103,6 +103,8 @@ def load(build_if_missing: bool = True):
     lib.rips_result_threshold.restype = C.c_float
     lib.rips_result_stats.argtypes = [vp, i32, i32, C.POINTER(Stats)]
     lib.rips_result_stats.restype = C.c_int
+    lib.rips_result_all_stats.argtypes = [vp, C.POINTER(Stats), fp]
+    lib.rips_result_all_stats.restype = C.c_int
     lib.rips_result_phase_ms.argtypes = [vp, fp, i32]
     lib.rips_result_phase_ms.restype = i32
     lib.rips_result_free.argtypes = [vp]

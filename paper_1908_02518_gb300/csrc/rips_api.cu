@@ -74,13 +74,17 @@ static int grow_keep(Buf& b, size_t bytes, size_t keep, cudaStream_t s) {
   return RIPS_OK;
 }
 
+// w.pin holds at least `bytes` (its contents do not survive growth)
+struct Workspace;
+static int ensure_pin(Workspace& w, size_t bytes);
+
 template <typename T>
 static T* P(Buf& b) {
   return (T*)b.p;
 }
 
 struct HostPinned {
-  uint32_t u32[16];
+  uint32_t u32[32];  // [16..31]: the reduction's control words
   unsigned long long u64[16 * (MAX_DIM + 1)];
   float f32[4];
 };
@@ -102,6 +106,8 @@ struct Workspace {
   Buf nrank, nkey, nkey_alt, nval, nval_alt, cursor;  // neighbour lists of a sparse input
   size_t r_cap = 0;
   HostPinned* pinned = nullptr;
+  unsigned char* pin = nullptr;  // pinned staging for what a call reads back (grow-only)
+  size_t pin_cap = 0;
   cudaEvent_t tev[16] = {};
   bool events = false;
   // per-kernel-class timing (enabled by rips_set_kernel_timing)
@@ -109,6 +115,21 @@ struct Workspace {
   std::vector<int> kev_class;         // class of each pair
   size_t kev_used = 0;                // pairs in use for the current call
 };
+
+static int ensure_pin(Workspace& w, size_t bytes) {
+  if (bytes <= w.pin_cap) return RIPS_OK;
+  if (w.pin) cudaFreeHost(w.pin);
+  w.pin = nullptr;
+  w.pin_cap = 0;
+  const size_t want = bytes + bytes / 2 + 4096;
+  if (cudaMallocHost((void**)&w.pin, want) != cudaSuccess) {
+    cudaGetLastError();
+    w.pin = nullptr;
+    return RIPS_ERR_OOM;
+  }
+  w.pin_cap = want;
+  return RIPS_OK;
+}
 
 static bool g_kernel_timing = false;
 
@@ -296,6 +317,8 @@ struct BatchOut {
   float kernel_ms[RIPS_KERNEL_CLASSES] = {};
   int64_t kernel_regions[RIPS_KERNEL_CLASSES] = {};
   uint32_t nbars = 0;
+  bool ordered = false;  // the bars are in canonical order in w.bars_alt and at `bars` (w.pin)
+  const rips_bar_t* bars = nullptr;
 };
 
 int sync_read(Workspace& w, cudaStream_t s) {
@@ -398,9 +421,14 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
     }
     CK(cudaMemcpyAsync(&hp->u32[0], w.ecount.p, 4, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(&hp->u32[1], w.err.p, 4, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(ccount.data(), w.ccounts.p, (size_t)C * 4, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(ci.data(), dclouds, (size_t)C * sizeof(CloudInfo), cudaMemcpyDeviceToHost, s));
+    CR(ensure_pin(w, (size_t)C * (sizeof(CloudInfo) + 4)));
+    CloudInfo* hci = (CloudInfo*)w.pin;
+    uint32_t* hcc = (uint32_t*)(hci + C);
+    CK(cudaMemcpyAsync(hcc, w.ccounts.p, (size_t)C * 4, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(hci, dclouds, (size_t)C * sizeof(CloudInfo), cudaMemcpyDeviceToHost, s));
     CR(sync_read(w, s));
+    ccount.assign(hcc, hcc + C);
+    ci.assign(hci, hci + C);
   } else {
     // the edges within the threshold, grown and listed again if the room was short
     for (int attempt = 0; attempt < 8; ++attempt) {
@@ -451,63 +479,6 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
   }
   const uint64_t* keys = alt ? P<uint64_t>(w.ekeys_alt) : P<uint64_t>(w.ekeys);
 
-  CR(ensure(w.eflags, (size_t)(m + 1) * 4));
-  CR(ensure(w.erank, (size_t)(m + 1) * 4));
-  CR(ensure(w.rvalue, (size_t)(m + 1) * 4));
-  if (!sp) CR(ensure(w.R, RR * 4));
-  CR(ensure(w.deg, (size_t)(N + 2) * 4));
-  {
-    KTimer kt(w, RIPS_K_PROLOGUE, s);
-    CK(launch_assign_ranks(keys, m, eb, P<uint32_t>(w.eflags), (uint32_t*)w.sorttmp.p, P<uint32_t>(w.erank),
-                           P<float>(w.rvalue), &P<uint32_t>(w.ecount)[1], s));
-    CK(cudaMemsetAsync(w.deg.p, 0, (size_t)(N + 2) * 4, s));
-    if (!sp) {
-      CK(cudaMemsetAsync(w.R.p, 0xFF, RR * 4, s));
-      CK(launch_fill_rank_matrix(keys, P<uint32_t>(w.erank), m, eb, dclouds, P<uint32_t>(w.R), s));
-      CK(launch_neighbor_counts(P<uint32_t>(w.R), dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, P<uint32_t>(w.deg),
-                                &P<uint32_t>(w.ecount)[3], s));
-    } else {
-      CK(cudaMemsetAsync((char*)w.ecount.p + 12, 0, 4, s));
-      CK(launch_sparse_degrees(keys, m, eb, P<uint32_t>(w.deg), s));
-      CK(launch_max(P<uint32_t>(w.deg), (uint32_t)N, &P<uint32_t>(w.ecount)[3], s));
-    }
-    CK(launch_exclusive_scan(P<uint32_t>(w.deg), P<uint32_t>(w.deg), (uint32_t)N + 1, w.sorttmp.p,
-                             &P<uint32_t>(w.ecount)[2], s));
-  }
-  CK(cudaMemcpyAsync(&hp->u32[2], (char*)w.ecount.p + 4, 12, cudaMemcpyDeviceToHost, s));
-  CR(sync_read(w, s));
-  const uint32_t num_ranks = hp->u32[2];
-  const uint32_t nbr_total = hp->u32[3];
-  const uint32_t max_deg = hp->u32[4];
-  CR(ensure(w.nbr, (size_t)nbr_total * 4 + 4));
-  CR(ensure(w.binom, (size_t)(kmax + 1) * (n_max + 1) * 8));
-  if (sp) {  // both directions of every edge with its rank, sorted into decreasing neighbour order
-    const uint32_t q = nbr_total;
-    CR(ensure(w.nrank, (size_t)q * 4 + 4));
-    CR(ensure(w.nkey, (size_t)q * 8 + 8));
-    CR(ensure(w.nkey_alt, (size_t)q * 8 + 8));
-    CR(ensure(w.nval, (size_t)q * 4 + 4));
-    CR(ensure(w.nval_alt, (size_t)q * 4 + 4));
-    CR(ensure(w.cursor, (size_t)N * 4 + 4));
-    CR(ensure(w.sorttmp, std::max(w.sorttmp.cap, sort_temp_bytes(q))));
-    KTimer kt(w, RIPS_K_PROLOGUE, s);
-    CK(cudaMemsetAsync(w.cursor.p, 0, (size_t)N * 4, s));
-    CK(launch_sparse_fill(keys, P<uint32_t>(w.erank), m, eb, P<uint32_t>(w.deg), P<uint32_t>(w.cursor),
-                          P<uint64_t>(w.nkey), P<uint32_t>(w.nval), s));
-    bool nalt = false;
-    CK(radix_sort_u64(P<uint64_t>(w.nkey), P<uint64_t>(w.nkey_alt), P<uint32_t>(w.nval), P<uint32_t>(w.nval_alt), q,
-                      32 + bit_width64((uint64_t)n_max), w.sorttmp.p, w.sorttmp.cap, &nalt, s));
-    CK(launch_sparse_unpack(nalt ? P<uint64_t>(w.nkey_alt) : P<uint64_t>(w.nkey),
-                            nalt ? P<uint32_t>(w.nval_alt) : P<uint32_t>(w.nval), q, P<uint32_t>(w.nbr),
-                            P<uint32_t>(w.nrank), s));
-    CK(launch_binomial_table(P<uint64_t>(w.binom), n_max, kmax, s));
-  } else {
-    KTimer kt(w, RIPS_K_PROLOGUE, s);
-    CK(launch_neighbor_fill(P<uint32_t>(w.R), dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, P<uint32_t>(w.deg),
-                            P<uint32_t>(w.nbr), s));
-    CK(launch_binomial_table(P<uint64_t>(w.binom), n_max, kmax, s));
-  }
-
   // ---------------- H0
   CR(grow_keep(w.bars, ((size_t)N + 16) * sizeof(rips_bar_t), 0, s));
   CR(ensure(w.inforest, (size_t)m + 1));
@@ -532,6 +503,7 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       CR(ensure(w.gtop, (size_t)n * 4));
       CR(ensure(w.fpos, (size_t)n * 4));
       CR(ensure(w.nf, 16));
+      CR(ensure(w.eflags, (size_t)(m + 1) * 4));
       CK(run_h0_large(n, keys, m, eb, P<uint32_t>(w.eu), P<uint32_t>(w.ev), P<uint32_t>(w.comp), P<uint32_t>(w.best),
                       P<uint32_t>(w.parent), P<uint8_t>(w.inforest), P<uint32_t>(w.eflags), P<uint32_t>(w.fpos),
                       w.sorttmp.p, P<uint32_t>(w.nf), P<uint32_t>(w.gtop), P<rips_bar_t>(w.bars),
@@ -539,10 +511,97 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
                       s));
     }
   }
+
+  if (dim_max > 0) {  // ranks, rank matrix and neighbour lists: for the simplices beyond the edges
+    CR(ensure(w.eflags, (size_t)(m + 1) * 4));
+    CR(ensure(w.erank, (size_t)(m + 1) * 4));
+    CR(ensure(w.rvalue, (size_t)(m + 1) * 4));
+    if (!sp) CR(ensure(w.R, RR * 4));
+    CR(ensure(w.deg, (size_t)(N + 2) * 4));
+    {
+      KTimer kt(w, RIPS_K_PROLOGUE, s);
+      CK(launch_assign_ranks(keys, m, eb, P<uint32_t>(w.eflags), (uint32_t*)w.sorttmp.p, P<uint32_t>(w.erank),
+                             P<float>(w.rvalue), &P<uint32_t>(w.ecount)[1], s));
+      CK(cudaMemsetAsync(w.deg.p, 0, (size_t)(N + 2) * 4, s));
+      if (!sp) {
+        CK(cudaMemsetAsync(w.R.p, 0xFF, RR * 4, s));
+        CK(launch_fill_rank_matrix(keys, P<uint32_t>(w.erank), m, eb, dclouds, P<uint32_t>(w.R), s));
+        CK(launch_neighbor_counts(P<uint32_t>(w.R), dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, P<uint32_t>(w.deg),
+                                  &P<uint32_t>(w.ecount)[3], s));
+      } else {
+        CK(cudaMemsetAsync((char*)w.ecount.p + 12, 0, 4, s));
+        CK(launch_sparse_degrees(keys, m, eb, P<uint32_t>(w.deg), s));
+        CK(launch_max(P<uint32_t>(w.deg), (uint32_t)N, &P<uint32_t>(w.ecount)[3], s));
+      }
+      CK(launch_exclusive_scan(P<uint32_t>(w.deg), P<uint32_t>(w.deg), (uint32_t)N + 1, w.sorttmp.p,
+                               &P<uint32_t>(w.ecount)[2], s));
+    }
+    // the number of ranks and the longest list: read at the next wait
+    CK(cudaMemcpyAsync(&hp->u32[2], (char*)w.ecount.p + 4, 12, cudaMemcpyDeviceToHost, s));
+    const uint32_t nbr_total = 2 * m;  // every edge is in two lists
+    CR(ensure(w.nbr, (size_t)nbr_total * 4 + 4));
+    CR(ensure(w.binom, (size_t)(kmax + 1) * (n_max + 1) * 8));
+    if (sp) {  // both directions of every edge with its rank, sorted into decreasing neighbour order
+      const uint32_t q = nbr_total;
+      CR(ensure(w.nrank, (size_t)q * 4 + 4));
+      CR(ensure(w.nkey, (size_t)q * 8 + 8));
+      CR(ensure(w.nkey_alt, (size_t)q * 8 + 8));
+      CR(ensure(w.nval, (size_t)q * 4 + 4));
+      CR(ensure(w.nval_alt, (size_t)q * 4 + 4));
+      CR(ensure(w.cursor, (size_t)N * 4 + 4));
+      CR(ensure(w.sorttmp, std::max(w.sorttmp.cap, sort_temp_bytes(q))));
+      KTimer kt(w, RIPS_K_PROLOGUE, s);
+      CK(cudaMemsetAsync(w.cursor.p, 0, (size_t)N * 4, s));
+      CK(launch_sparse_fill(keys, P<uint32_t>(w.erank), m, eb, P<uint32_t>(w.deg), P<uint32_t>(w.cursor),
+                            P<uint64_t>(w.nkey), P<uint32_t>(w.nval), s));
+      bool nalt = false;
+      CK(radix_sort_u64(P<uint64_t>(w.nkey), P<uint64_t>(w.nkey_alt), P<uint32_t>(w.nval), P<uint32_t>(w.nval_alt), q,
+                        32 + bit_width64((uint64_t)n_max), w.sorttmp.p, w.sorttmp.cap, &nalt, s));
+      CK(launch_sparse_unpack(nalt ? P<uint64_t>(w.nkey_alt) : P<uint64_t>(w.nkey),
+                              nalt ? P<uint32_t>(w.nval_alt) : P<uint32_t>(w.nval), q, P<uint32_t>(w.nbr),
+                              P<uint32_t>(w.nrank), s));
+      CK(launch_binomial_table(P<uint64_t>(w.binom), n_max, kmax, s));
+    } else {
+      KTimer kt(w, RIPS_K_PROLOGUE, s);
+      CK(launch_neighbor_fill(P<uint32_t>(w.R), dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, P<uint32_t>(w.deg),
+                              P<uint32_t>(w.nbr), s));
+      CK(launch_binomial_table(P<uint64_t>(w.binom), n_max, kmax, s));
+    }
+  }
   if (w.events) CK(cudaEventRecord(w.tev[1], s));
 
   // ---------------- dimensions 1..dim_max
+  // Bits and range of a diameter rank: ranks number distinct lengths, so the edge count bounds them; only when keys of
+  // that many bits would not fit is the number of ranks read back first.
+  const auto keys_fit = [&](int rb) {
+    for (int d = 1; d <= dim_max; ++d) {
+      const int col = bits_of_count(host_binom(n_max, d + 1)), row = bits_of_count(host_binom(n_max, d + 2));
+      if (rb + row > 63 || cb + rb + col > 64 || cb + row > 64) return false;
+    }
+    return true;
+  };
+  uint32_t num_ranks = m;
+  if (dim_max > 0 && !keys_fit(bit_width64(m ? m - 1 : 0))) {
+    CR(sync_read(w, s));
+    num_ranks = hp->u32[2];
+  }
   const int rank_bits = bit_width64(num_ranks ? num_ranks - 1 : 0);
+  // A result of at most `most` bars, few enough for one block to put in order: ordered with the count on the device
+  // and read back with the counters in the wait that ends the call.  Three waits less than a read-back each of the
+  // ranks, the bar count and the bars: 100 points, dimension 1: 0.81 -> 0.76 ms; 33 points: 0.37 -> 0.32 ms.
+  const unsigned long long* hstats = nullptr;  // counters on the host (w.pin)
+  const auto read_ordered = [&](uint64_t most) -> int {
+    const size_t bytes = (size_t)most * sizeof(rips_bar_t);
+    CR(ensure(w.bars_alt, bytes));
+    CR(ensure_pin(w, bytes + (size_t)C * SPC * 8));
+    CK(launch_bar_order_small(P<rips_bar_t>(w.bars), P<rips_bar_t>(w.bars_alt), (uint32_t)most, P<uint32_t>(w.nbars), s));
+    CK(cudaMemcpyAsync(w.pin, w.bars_alt.p, bytes, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(w.pin + bytes, dstats, (size_t)C * SPC * 8, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(&hp->u32[11], w.nbars.p, 4, cudaMemcpyDeviceToHost, s));
+    out.bars = (const rips_bar_t*)w.pin;
+    hstats = (const unsigned long long*)(w.pin + bytes);
+    return RIPS_OK;
+  };
   uint32_t ns_prev = 0;  // size of the (d-1)-simplex list in sidx[cur^1]
   int prev_col_bits = 0;
   int cur = 0;
@@ -679,6 +738,7 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
     if (blocks < 1) return RIPS_ERR_CUDA;
     CR(ensure(w.wide, wide_ctx_bytes(blocks)));
     uint32_t slice = 32;
+    const uint32_t max_deg = hp->u32[4];  // read with the ranks' number, before this dimension's wait
     while (slice < max_deg + 1) slice <<= 1;
     // The arena holds the working columns' tables and lists and the stored
     // columns; an arena that proves too small costs a rerun of the dimension with
@@ -739,14 +799,20 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
         KTimer kt(w, RIPS_K_REDUCE, s);
         CK(launch_reduction(a, rs, blocks, counts, s));
       }
-      CK(cudaMemcpyAsync(&hp->u32[6], counts + 6, 4, cudaMemcpyDeviceToHost, s));
+      {
+        KTimer kt(w, RIPS_K_READOUT, s);
+        CK(launch_readout(a, rs, P<float>(w.rvalue), P<rips_bar_t>(w.bars), P<uint32_t>(w.nbars),
+                          (uint32_t)(w.bars.cap / sizeof(rips_bar_t)), st, SPC, s));
+      }
+      if (w.events && d + 1 < 16) CK(cudaEventRecord(w.tev[d + 1], s));
+      const uint64_t most = (uint64_t)hp->u32[10] + M;  // bars so far and one per column
+      const bool last = d == dim_max && most <= bar_order_small_most();
+      if (last) CR(read_ordered(most));
+      CK(cudaMemcpyAsync(&hp->u32[16], counts, 64, cudaMemcpyDeviceToHost, s));
       CK(cudaMemcpyAsync(&hp->u32[8], w.err.p, 4, cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(&hp->u64[1], rs.steps, 16, cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(&hp->u64[3], rs.added, 8, cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(&hp->u32[9], counts + 7, 4, cudaMemcpyDeviceToHost, s));
       CR(sync_read(w, s));
       if (hp->u32[8] & ERRF_ARENA) {
-        // start this dimension's reduction over with a larger arena
+        // start this dimension's reduction over with a larger arena (the readout of a failed one writes nothing)
         CK(cudaMemsetAsync(w.err.p, 0, 4, s));
         rcap *= 8;
         continue;
@@ -754,18 +820,18 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       if (int e = map_device_error(hp->u32[8])) return e;
       out.stats.resize((size_t)C * (dim_max + 1));
       // rounds and steps are properties of the whole batch's reduction
+      const uint32_t* hc = &hp->u32[16];
+      unsigned long long hl[8];
+      memcpy(hl, hc, sizeof(hl));
       for (int c = 0; c < C; ++c) {
-        out.stats[(size_t)c * (dim_max + 1) + d].rounds = hp->u32[6];
-        out.stats[(size_t)c * (dim_max + 1) + d].reduction_steps = (int64_t)hp->u64[1];
-        out.stats[(size_t)c * (dim_max + 1) + d].longest_chain = hp->u32[9];
-        out.stats[(size_t)c * (dim_max + 1) + d].compacted_entries = (int64_t)hp->u64[2];
-        out.stats[(size_t)c * (dim_max + 1) + d].added_entries = (int64_t)hp->u64[3];
+        rips_stats_t& q = out.stats[(size_t)c * (dim_max + 1) + d];
+        q.rounds = hc[6];
+        q.reduction_steps = (int64_t)hl[4];
+        q.longest_chain = hc[7];
+        q.compacted_entries = (int64_t)hl[5];
+        q.added_entries = (int64_t)hl[7];
       }
-      {
-        KTimer kt(w, RIPS_K_READOUT, s);
-        CK(launch_readout(a, rs, P<float>(w.rvalue), P<rips_bar_t>(w.bars), P<uint32_t>(w.nbars),
-                          (uint32_t)(w.bars.cap / sizeof(rips_bar_t)), st, SPC, s));
-      }
+      out.ordered = last;
       done = true;
     }
     if (!done) return RIPS_ERR_OOM;
@@ -776,20 +842,27 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
     ns_prev = nsd;
     prev_col_bits = a.col_bits;
     cur ^= 1;
-    if (w.events && d + 1 < 16) CK(cudaEventRecord(w.tev[d + 1], s));
   }
 
   // statistics and bar count
-  std::vector<unsigned long long> hstats((size_t)C * SPC);
-  CK(cudaMemcpyAsync(hstats.data(), dstats, (size_t)C * SPC * 8, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(&hp->u32[11], w.nbars.p, 4, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(&hp->u32[12], w.err.p, 4, cudaMemcpyDeviceToHost, s));
-  CR(sync_read(w, s));
-  if (int e = map_device_error(hp->u32[12])) return e;
+  if (!out.ordered) {
+    out.ordered = dim_max == 0 && N <= bar_order_small_most();
+    if (out.ordered) {
+      CR(read_ordered(N));
+    } else {
+      CR(ensure_pin(w, (size_t)C * SPC * 8));
+      hstats = (const unsigned long long*)w.pin;
+      CK(cudaMemcpyAsync(w.pin, dstats, (size_t)C * SPC * 8, cudaMemcpyDeviceToHost, s));
+      CK(cudaMemcpyAsync(&hp->u32[11], w.nbars.p, 4, cudaMemcpyDeviceToHost, s));
+    }
+    CK(cudaMemcpyAsync(&hp->u32[8], w.err.p, 4, cudaMemcpyDeviceToHost, s));
+    CR(sync_read(w, s));
+  }
+  if (int e = map_device_error(hp->u32[8])) return e;
   out.nbars = hp->u32[11];
   out.stats.resize((size_t)C * (dim_max + 1));
   for (int c = 0; c < C; ++c) {
-    const unsigned long long* q0 = hstats.data() + (size_t)c * SPC;
+    const unsigned long long* q0 = hstats + (size_t)c * SPC;
     rips_stats_t& s0 = out.stats[(size_t)c * (dim_max + 1)];
     s0.simplices = ns[c];
     s0.columns = ns[c];
@@ -833,20 +906,39 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
 }
 
 // canonical order on the device and copy to the host
-int finish_bars(Workspace& w, uint32_t nb, int simplex_bits, int group_bits, cudaStream_t s,
+int finish_bars(Workspace& w, const BatchOut& bo, int simplex_bits, int group_bits, cudaStream_t s,
                 std::vector<rips_bar_t>& host) {
-  host.resize(nb);
+  const uint32_t nb = bo.nbars;
+  if (bo.ordered) {  // done with the last read-back
+    host.assign(bo.bars, bo.bars + nb);
+    return RIPS_OK;
+  }
+  host.clear();
   if (nb == 0) return RIPS_OK;
   CR(ensure(w.bars_alt, (size_t)nb * sizeof(rips_bar_t)));
-  CR(ensure(w.bk0, (size_t)nb * 8));
-  CR(ensure(w.bk1, (size_t)nb * 8));
-  CR(ensure(w.bp0, (size_t)nb * 4));
-  CR(ensure(w.bp1, (size_t)nb * 4));
-  CR(ensure(w.bartmp, bar_order_temp_bytes(nb)));
-  CK(launch_bar_order(P<rips_bar_t>(w.bars), P<rips_bar_t>(w.bars_alt), nb, P<uint64_t>(w.bk0), P<uint64_t>(w.bk1),
-                      P<uint32_t>(w.bp0), P<uint32_t>(w.bp1), w.bartmp.p, w.bartmp.cap, simplex_bits, group_bits, s));
-  CK(cudaMemcpyAsync(host.data(), w.bars_alt.p, (size_t)nb * sizeof(rips_bar_t), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  if (nb <= bar_order_small_most()) {
+    CK(launch_bar_order_small(P<rips_bar_t>(w.bars), P<rips_bar_t>(w.bars_alt), nb, P<uint32_t>(w.nbars), s));
+  } else {
+    CR(ensure(w.bk0, (size_t)nb * 8));
+    CR(ensure(w.bk1, (size_t)nb * 8));
+    CR(ensure(w.bp0, (size_t)nb * 4));
+    CR(ensure(w.bp1, (size_t)nb * 4));
+    CR(ensure(w.bartmp, bar_order_temp_bytes(nb)));
+    CK(launch_bar_order(P<rips_bar_t>(w.bars), P<rips_bar_t>(w.bars_alt), nb, P<uint64_t>(w.bk0), P<uint64_t>(w.bk1),
+                        P<uint32_t>(w.bp0), P<uint32_t>(w.bp1), w.bartmp.p, w.bartmp.cap, simplex_bits, group_bits, s));
+  }
+  // through pinned memory up to 8 MB (it stays with the workspace), longer results straight to where they go
+  const size_t bytes = (size_t)nb * sizeof(rips_bar_t);
+  if (bytes <= ((size_t)8 << 20)) {
+    CR(ensure_pin(w, bytes));
+    CK(cudaMemcpyAsync(w.pin, w.bars_alt.p, bytes, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    host.assign((const rips_bar_t*)w.pin, (const rips_bar_t*)w.pin + nb);
+  } else {
+    host.resize(nb);
+    CK(cudaMemcpyAsync(host.data(), w.bars_alt.p, bytes, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+  }
   return RIPS_OK;
 }
 
@@ -880,7 +972,7 @@ int barcodes_locked(Workspace& w, const float* dD, int64_t n, int32_t dim_max, f
   int rc = run_batch(w, dD, ns, dim_max, threshold, p, s, bo);
   if (rc == RIPS_OK) {
     const int sbits = std::max(1, bit_width64(host_binom((uint64_t)n, dim_max + 1)));
-    rc = finish_bars(w, bo.nbars, sbits, 0, s, r->bars);
+    rc = finish_bars(w, bo, sbits, 0, s, r->bars);
   }
   if (rc != RIPS_OK) {
     delete r;
@@ -907,7 +999,7 @@ int sparse_locked(Workspace& w, const SparseIn& sp, int64_t n, int32_t dim_max, 
   int rc = run_batch(w, nullptr, ns, dim_max, threshold, p, s, bo, &sp);
   if (rc == RIPS_OK) {
     const int sbits = std::max(1, bit_width64(host_binom((uint64_t)n, dim_max + 1)));
-    rc = finish_bars(w, bo.nbars, sbits, 0, s, r->bars);
+    rc = finish_bars(w, bo, sbits, 0, s, r->bars);
   }
   if (rc != RIPS_OK) {
     delete r;
@@ -980,7 +1072,7 @@ int batched_locked(Workspace& w, const float* d_points, const int64_t* offsets, 
   if (rc == RIPS_OK) rc = run_batch(w, P<float>(w.cdist), ns, dim_max, threshold, p, s, bo);
   if (rc == RIPS_OK) {
     const int sbits = std::max(1, bit_width64(host_binom((uint64_t)nmax, dim_max + 1)));
-    rc = finish_bars(w, bo.nbars, sbits, std::max(1, bit_width64((uint64_t)batch)), s, r->bars);
+    rc = finish_bars(w, bo, sbits, std::max(1, bit_width64((uint64_t)batch)), s, r->bars);
   }
   if (rc != RIPS_OK) {
     delete r;
@@ -1048,7 +1140,7 @@ int batched_dists_locked(Workspace& w, const float* const* d_dists, const int64_
   if (rc == RIPS_OK) rc = run_batch(w, P<float>(w.cdist), ns, dim_max, threshold, p, s, bo);
   if (rc == RIPS_OK) {
     const int sbits = std::max(1, bit_width64(host_binom((uint64_t)nmax, dim_max + 1)));
-    rc = finish_bars(w, bo.nbars, sbits, std::max(1, bit_width64((uint64_t)batch)), s, r->bars);
+    rc = finish_bars(w, bo, sbits, std::max(1, bit_width64((uint64_t)batch)), s, r->bars);
   }
   if (rc != RIPS_OK) {
     delete r;
@@ -1132,6 +1224,9 @@ void release_plan(PlanState& pl) {
                 &w.bars, &w.bars_alt, &w.bk0, &w.bk1, &w.bp0, &w.bp1, &w.bartmp, &w.nbars, &w.stats,
                 &w.bwd_bars, &w.bwd_off, &w.cdist, &w.clouds, &w.tileoff, &w.vcloud, &w.ccounts, &pl.clouds0};
   for (Buf* b : all) release(*b);
+  if (w.pin) cudaFreeHost(w.pin);
+  w.pin = nullptr;
+  w.pin_cap = 0;
 }
 
 int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k, float threshold, uint32_t p,
@@ -1378,19 +1473,35 @@ int plan_run(PlanState& pl, const float* d_points, cudaStream_t s) {
 int plan_result(PlanState& pl, cudaStream_t s, rips_result_t** out) {
   Workspace& w = pl.w;
   const int C = pl.C;
+  // the run's end: on this stream, and on any other that waits with the default stream
+  uint32_t err = 0;
   CK(cudaStreamSynchronize(s));
-  uint32_t err = 0, nbars = 0, counts[32] = {};
-  unsigned long long lists[16] = {};
-  std::vector<unsigned long long> hst((size_t)C * PLAN_SPC);
-  std::vector<CloudInfo> ci(C);
   CK(cudaMemcpy(&err, w.err.p, 4, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(&nbars, w.nbars.p, 4, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(counts, w.lists.p, 128, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(lists, w.lists.p, 128, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(hst.data(), w.stats.p, hst.size() * 8, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(ci.data(), w.clouds.p, (size_t)C * sizeof(CloudInfo), cudaMemcpyDeviceToHost));
   if (err & ERRF_ARENA) return RIPS_ERR_OOM;  // the plan's arena is fixed: make the plan with a larger one
   if (int e = map_device_error(err)) return e;
+  // one more wait: counters and statistics, and as many of the bars, in order, as the small sort takes
+  const uint32_t most = (uint32_t)std::min<size_t>(bar_order_small_most(), w.bars.cap / sizeof(rips_bar_t));
+  const size_t bars_at = 256, st_at = bars_at + (size_t)most * sizeof(rips_bar_t),
+               ci_at = st_at + (size_t)C * PLAN_SPC * 8;
+  CR(ensure_pin(w, ci_at + (size_t)C * sizeof(CloudInfo)));
+  CR(ensure(w.bars_alt, (size_t)most * sizeof(rips_bar_t)));
+  CK(launch_bar_order_small(P<rips_bar_t>(w.bars), P<rips_bar_t>(w.bars_alt), most, P<uint32_t>(w.nbars), s));
+  CK(cudaMemcpyAsync(w.pin, w.lists.p, 64, cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(w.pin + 64, w.nbars.p, 4, cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(w.pin + bars_at, w.bars_alt.p, (size_t)most * sizeof(rips_bar_t), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(w.pin + st_at, w.stats.p, (size_t)C * PLAN_SPC * 8, cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(w.pin + ci_at, w.clouds.p, (size_t)C * sizeof(CloudInfo), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  uint32_t counts[17];
+  unsigned long long lists[8];
+  memcpy(counts, w.pin, sizeof(counts));
+  memcpy(lists, w.pin, sizeof(lists));
+  BatchOut bo;
+  bo.nbars = counts[16];
+  bo.ordered = bo.nbars <= most;
+  bo.bars = (const rips_bar_t*)(w.pin + bars_at);
+  const unsigned long long* hst = (const unsigned long long*)(w.pin + st_at);
+  const CloudInfo* ci = (const CloudInfo*)(w.pin + ci_at);
   rips_result* r = new (std::nothrow) rips_result();
   if (!r) return RIPS_ERR_OOM;
   r->clouds = C;
@@ -1402,7 +1513,7 @@ int plan_result(PlanState& pl, cudaStream_t s, rips_result_t** out) {
   r->stats.resize((size_t)C * 2);
   for (int c = 0; c < C; ++c) {
     r->thresholds[c] = ci[c].t_eff;
-    const unsigned long long* q0 = hst.data() + (size_t)c * PLAN_SPC;
+    const unsigned long long* q0 = hst + (size_t)c * PLAN_SPC;
     rips_stats_t& s0 = r->stats[(size_t)c * 2];
     s0.simplices = pl.ns[c];
     s0.columns = pl.ns[c];
@@ -1427,7 +1538,7 @@ int plan_result(PlanState& pl, cudaStream_t s, rips_result_t** out) {
     sd.added_entries = (int64_t)lists[7];
   }
   const int sbits = std::max(1, bit_width64(host_binom((uint64_t)pl.n_max, 2)));
-  const int rc = finish_bars(w, nbars, sbits, std::max(1, bit_width64((uint64_t)C)), s, r->bars);
+  const int rc = finish_bars(w, bo, sbits, std::max(1, bit_width64((uint64_t)C)), s, r->bars);
   if (rc != RIPS_OK) {
     delete r;
     return rc;
@@ -1580,6 +1691,13 @@ RIPS_API float rips_result_threshold(const rips_result_t* r, int32_t cloud) {
 RIPS_API int rips_result_stats(const rips_result_t* r, int32_t cloud, int32_t dim, rips_stats_t* out) {
   if (!r || !out || cloud < 0 || cloud >= r->clouds || dim < 0 || dim > r->dim_max) return RIPS_ERR_BAD_ARG;
   *out = r->stats[(size_t)cloud * (r->dim_max + 1) + dim];
+  return RIPS_OK;
+}
+
+RIPS_API int rips_result_all_stats(const rips_result_t* r, rips_stats_t* stats, float* thresholds) {
+  if (!r) return RIPS_ERR_BAD_ARG;
+  if (stats) memcpy(stats, r->stats.data(), r->stats.size() * sizeof(rips_stats_t));
+  if (thresholds) memcpy(thresholds, r->thresholds.data(), r->thresholds.size() * sizeof(float));
   return RIPS_OK;
 }
 

@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(256) test_kernel(DimArgs a, const uint64_t* __
 __global__ void readout_kernel(DimArgs a, RedState s, const float* __restrict__ rank_value,
                                rips_bar_t* __restrict__ bars, uint32_t* __restrict__ nbars, uint32_t bar_cap,
                                unsigned long long* __restrict__ stats, int st_stride) {
+  if (*s.err) return;  // the reduction did not end: no pivots to read, and the call fails or starts it over
   const uint32_t ncols = s.ncols_dev ? *s.ncols_dev : s.ncols;
   for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < ncols; j += gridDim.x * blockDim.x) {
     uint64_t idx;

@@ -28,14 +28,19 @@ __global__ void bar_key_kernel(const rips_bar_t* __restrict__ bars, const uint32
   keys[i] = k;
 }
 
-// Up to SMALL_BARS bars: one block sorts their indices by the same three keys
+// Up to SMALL_BARS bars (their number read on the device): one block sorts their indices by the same three keys
 // (group, birth and death, birth simplex; no two bars share all three) with a
 // bitonic network in shared memory and gathers them, in one launch.
 constexpr uint32_t SMALL_BARS = 2048;
 
-__global__ void __launch_bounds__(1024) bar_order_small_kernel(const rips_bar_t* __restrict__ bars, uint32_t n,
-                                                                uint32_t n2, rips_bar_t* __restrict__ out) {
+__global__ void __launch_bounds__(1024) bar_order_small_kernel(const rips_bar_t* __restrict__ bars, uint32_t most,
+                                                                const uint32_t* __restrict__ count,
+                                                                rips_bar_t* __restrict__ out) {
   extern __shared__ uint64_t sm[];
+  const uint32_t n = *count;
+  if (n > most) return;  // more than there is room for: the host sorts them otherwise
+  uint32_t n2 = 2;
+  while (n2 < n) n2 <<= 1;
   uint64_t* k2 = sm;           // cloud and dimension
   uint64_t* k1 = sm + n2;      // birth and death bits
   uint64_t* k0 = sm + 2 * n2;  // birth simplex
@@ -81,30 +86,33 @@ __global__ void gather_bars_kernel(const rips_bar_t* __restrict__ in, const uint
 
 }  // namespace
 
+uint32_t bar_order_small_most() { return SMALL_BARS; }
+
+cudaError_t launch_bar_order_small(const rips_bar_t* bars, rips_bar_t* bars_alt, uint32_t most, const uint32_t* count,
+                                   cudaStream_t s) {
+  uint32_t n2 = 2;
+  while (n2 < most) n2 <<= 1;
+  static std::atomic<bool> opted[64];  // once per device (any thread)
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(bar_order_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(SMALL_BARS * 28));
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) opted[dev].store(true, std::memory_order_release);
+  }
+  bar_order_small_kernel<<<1, 1024, (size_t)n2 * 28, s>>>(bars, most, count, bars_alt);
+  note_launch();
+  return cudaGetLastError();
+}
+
 size_t bar_order_temp_bytes(uint32_t nb) { return sort_temp_bytes(nb); }
 
 cudaError_t launch_bar_order(rips_bar_t* bars, rips_bar_t* bars_alt, uint32_t nb, uint64_t* k0, uint64_t* k1,
                              uint32_t* p0, uint32_t* p1, void* tmp, size_t tmp_bytes, int simplex_bits,
                              int group_bits, cudaStream_t s) {
   if (nb == 0) return cudaSuccess;
-  if (nb <= SMALL_BARS) {
-    uint32_t n2 = 2;
-    while (n2 < nb) n2 <<= 1;
-    const size_t smem = (size_t)n2 * 28;
-    static std::atomic<bool> opted[64];  // once per device (any thread)
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
-      e = cudaFuncSetAttribute(bar_order_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(SMALL_BARS * 28));
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) opted[dev].store(true, std::memory_order_release);
-    }
-    bar_order_small_kernel<<<1, 1024, smem, s>>>(bars, nb, n2, bars_alt);
-    note_launch();
-    return cudaGetLastError();
-  }
   const int blocks = (int)((nb + 255) / 256);
   iota_kernel<<<blocks, 256, 0, s>>>(p0, nb);
   note_launch();

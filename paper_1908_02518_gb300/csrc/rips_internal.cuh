@@ -286,6 +286,11 @@ cudaError_t launch_readout(const DimArgs& a, const RedState& s, const float* ran
                            cudaStream_t st);
 
 // from rips_epilogue.cu
+// canonical order of up to `most` (<= bar_order_small_most()) bars, their number *count read on the device; nothing is
+// written when there are more
+uint32_t bar_order_small_most();
+cudaError_t launch_bar_order_small(const rips_bar_t* bars, rips_bar_t* bars_alt, uint32_t most, const uint32_t* count,
+                                   cudaStream_t s);
 cudaError_t launch_bar_order(rips_bar_t* bars, rips_bar_t* bars_alt, uint32_t nb, uint64_t* k0, uint64_t* k1,
                              uint32_t* p0, uint32_t* p1, void* tmp, size_t tmp_bytes, int simplex_bits,
                              int group_bits, cudaStream_t s);
