@@ -409,15 +409,27 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
   CK(cudaMemsetAsync(w.ecount.p, 0, 16, s));
   CK(cudaMemsetAsync(w.ccounts.p, 0, (size_t)(C + 1) * 4, s));
   std::vector<uint32_t> ccount(C);
+  // Edges that may be too many for the one-block sort are listed in index order, so that a radix sort leaves the index
+  // bits out; fewer are sorted by all bits in one launch, and placing them in any order takes one kernel instead of three.
+  const bool ordered = !sp && e_cap > SMALL_SORT;
   if (!sp) {
+    if (ordered) {
+      CR(ensure(w.deg, (size_t)(N + 2) * 4));
+      CR(ensure(w.sorttmp, scan_temp_bytes((uint32_t)N)));
+    }
     {
       KTimer kt(w, RIPS_K_PROLOGUE, s);
       CK(launch_cloud_vertices(dclouds, C, P<uint32_t>(w.vcloud), s));
       CK(launch_validate_rowmax(dD, dclouds, P<uint32_t>(w.tileoff), C, (uint32_t)tiles, P<uint32_t>(w.rowmax),
                                 P<uint32_t>(w.err), s));
       CK(launch_threshold(P<uint32_t>(w.rowmax), dclouds, C, threshold, s));
-      CK(launch_edge_keys(dD, dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, eb, P<uint64_t>(w.ekeys),
-                          P<uint32_t>(w.ecount), P<uint32_t>(w.ccounts), (uint32_t)e_cap, s));
+      if (ordered)
+        CK(launch_edge_keys_ordered(dD, dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, eb, P<uint64_t>(w.ekeys),
+                                    P<uint32_t>(w.deg), w.sorttmp.p, P<uint32_t>(w.ecount), P<uint32_t>(w.ccounts),
+                                    (uint32_t)e_cap, s));
+      else
+        CK(launch_edge_keys(dD, dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, eb, P<uint64_t>(w.ekeys),
+                            P<uint32_t>(w.ecount), P<uint32_t>(w.ccounts), (uint32_t)e_cap, s));
     }
     CK(cudaMemcpyAsync(&hp->u32[0], w.ecount.p, 4, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(&hp->u32[1], w.err.p, 4, cudaMemcpyDeviceToHost, s));
@@ -474,8 +486,8 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
   bool alt = false;
   {
     KTimer kt(w, RIPS_K_EDGE_SORT, s);
-    CK(radix_sort_u64(P<uint64_t>(w.ekeys), P<uint64_t>(w.ekeys_alt), nullptr, nullptr, m, cb + 32 + eb,
-                      w.sorttmp.p, w.sorttmp.cap, &alt, s));
+    CK(radix_sort_u64(P<uint64_t>(w.ekeys), P<uint64_t>(w.ekeys_alt), nullptr, nullptr, m, ordered ? eb : 0,
+                      cb + 32 + eb, w.sorttmp.p, w.sorttmp.cap, &alt, s));
   }
   const uint64_t* keys = alt ? P<uint64_t>(w.ekeys_alt) : P<uint64_t>(w.ekeys);
 
@@ -555,7 +567,7 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       CK(launch_sparse_fill(keys, P<uint32_t>(w.erank), m, eb, P<uint32_t>(w.deg), P<uint32_t>(w.cursor),
                             P<uint64_t>(w.nkey), P<uint32_t>(w.nval), s));
       bool nalt = false;
-      CK(radix_sort_u64(P<uint64_t>(w.nkey), P<uint64_t>(w.nkey_alt), P<uint32_t>(w.nval), P<uint32_t>(w.nval_alt), q,
+      CK(radix_sort_u64(P<uint64_t>(w.nkey), P<uint64_t>(w.nkey_alt), P<uint32_t>(w.nval), P<uint32_t>(w.nval_alt), q, 0,
                         32 + bit_width64((uint64_t)n_max), w.sorttmp.p, w.sorttmp.cap, &nalt, s));
       CK(launch_sparse_unpack(nalt ? P<uint64_t>(w.nkey_alt) : P<uint64_t>(w.nkey),
                               nalt ? P<uint32_t>(w.nval_alt) : P<uint32_t>(w.nval), q, P<uint32_t>(w.nbr),
@@ -709,7 +721,7 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
     bool calt = false;
     {
       KTimer kt(w, RIPS_K_COL_SORT, s);
-      CK(radix_sort_u64(P<uint64_t>(w.ckeys), P<uint64_t>(w.ckeys_alt), nullptr, nullptr, M,
+      CK(radix_sort_u64(P<uint64_t>(w.ckeys), P<uint64_t>(w.ckeys_alt), nullptr, nullptr, M, 0,
                         cb + rank_bits + a.col_bits, w.sorttmp.p, w.sorttmp.cap, &calt, s));
     }
     const uint64_t* ckeys = calt ? P<uint64_t>(w.ckeys_alt) : P<uint64_t>(w.ckeys);
@@ -1391,13 +1403,19 @@ int plan_run(PlanState& pl, const float* d_points, cudaStream_t s) {
   CK(launch_validate_rowmax(dD, dclouds, P<uint32_t>(w.tileoff), C, (uint32_t)pl.vtiles, P<uint32_t>(w.rowmax),
                             P<uint32_t>(w.err), s));
   CK(launch_threshold(P<uint32_t>(w.rowmax), dclouds, C, pl.threshold, s));
-  CK(launch_edge_keys(dD, dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, pl.eb, P<uint64_t>(w.ekeys),
-                      P<uint32_t>(w.ecount), P<uint32_t>(w.ccounts), (uint32_t)E, s));
+  const bool ordered = E > SMALL_SORT;  // as in a call without a plan
+  if (ordered)
+    CK(launch_edge_keys_ordered(dD, dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, pl.eb, P<uint64_t>(w.ekeys),
+                                P<uint32_t>(w.deg), w.sorttmp.p, P<uint32_t>(w.ecount), P<uint32_t>(w.ccounts),
+                                (uint32_t)E, s));
+  else
+    CK(launch_edge_keys(dD, dclouds, P<uint32_t>(w.vcloud), (uint32_t)N, pl.eb, P<uint64_t>(w.ekeys),
+                        P<uint32_t>(w.ecount), P<uint32_t>(w.ccounts), (uint32_t)E, s));
   CK(launch_cloud_edge_offsets(dclouds, P<uint32_t>(w.ccounts), C, s));
   CK(launch_pad_past_count(P<uint64_t>(w.ekeys), P<uint32_t>(w.ecount), E, s));
   bool alt = false;
   CK(radix_sort_u64(P<uint64_t>(w.ekeys), P<uint64_t>(w.ekeys_alt), nullptr, nullptr, (uint32_t)E,
-                    pl.cb + 32 + pl.eb, w.sorttmp.p, w.sorttmp.cap, &alt, s));
+                    ordered ? pl.eb : 0, pl.cb + 32 + pl.eb, w.sorttmp.p, w.sorttmp.cap, &alt, s));
   const uint64_t* keys = alt ? P<uint64_t>(w.ekeys_alt) : P<uint64_t>(w.ekeys);
   CK(launch_assign_ranks(keys, (uint32_t)E, pl.eb, P<uint32_t>(w.eflags), (uint32_t*)w.sorttmp.p,
                          P<uint32_t>(w.erank), P<float>(w.rvalue), &P<uint32_t>(w.ecount)[1], s));
@@ -1427,7 +1445,7 @@ int plan_run(PlanState& pl, const float* d_points, cudaStream_t s) {
   CK(launch_pad_past_count(P<uint64_t>(w.ckeys), P<uint32_t>(w.ccount), E, s));
   bool calt = false;
   CK(radix_sort_u64(P<uint64_t>(w.ckeys), P<uint64_t>(w.ckeys_alt), nullptr, nullptr, (uint32_t)E,
-                    pl.cb + a.rank_bits + a.col_bits, w.sorttmp.p, w.sorttmp.cap, &calt, s));
+                    0, pl.cb + a.rank_bits + a.col_bits, w.sorttmp.p, w.sorttmp.cap, &calt, s));
   CK(cudaMemsetAsync(w.tkeys[0].p, 0xFF, (size_t)pl.tcap * 8, s));
   CK(cudaMemsetAsync(w.tvals[0].p, 0xFF, (size_t)pl.tcap * 4, s));
   CK(cudaMemsetAsync(w.lists.p, 0, LISTS_BYTES, s));

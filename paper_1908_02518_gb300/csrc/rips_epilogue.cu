@@ -123,7 +123,7 @@ cudaError_t launch_bar_order(rips_bar_t* bars, rips_bar_t* bars_alt, uint32_t nb
     bar_key_kernel<<<blocks, 256, 0, s>>>(bars, perm, nb, which, k0);
     note_launch();
     bool alt = false;
-    cudaError_t e = radix_sort_u64(k0, k1, perm, perm_alt, nb, bits[which], tmp, tmp_bytes, &alt, s);
+    cudaError_t e = radix_sort_u64(k0, k1, perm, perm_alt, nb, 0, bits[which], tmp, tmp_bytes, &alt, s);
     if (e != cudaSuccess) return e;
     if (alt) {
       uint32_t* t = perm;

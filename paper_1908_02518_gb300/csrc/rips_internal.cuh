@@ -125,6 +125,10 @@ cudaError_t launch_threshold(const uint32_t* rowmax_bits, CloudInfo* clouds, int
 cudaError_t launch_edge_keys(const float* D, const CloudInfo* clouds, const uint32_t* vcloud, uint32_t nverts,
                              int edge_bits, uint64_t* keys, uint32_t* count, uint32_t* cloud_count, uint32_t cap,
                              cudaStream_t s);
+// the same keys in decreasing edge order; row_off: nverts words; scan_tmp: scan_temp_bytes(nverts)
+cudaError_t launch_edge_keys_ordered(const float* D, const CloudInfo* clouds, const uint32_t* vcloud, uint32_t nverts,
+                                     int edge_bits, uint64_t* keys, uint32_t* row_off, void* scan_tmp, uint32_t* count,
+                                     uint32_t* cloud_count, uint32_t cap, cudaStream_t s);
 cudaError_t launch_assign_ranks(const uint64_t* sorted_keys, uint32_t num_edges, int edge_bits, uint32_t* flags,
                                 uint32_t* scan_tmp, uint32_t* edge_rank, float* rank_value, uint32_t* num_ranks,
                                 cudaStream_t s);
@@ -160,11 +164,15 @@ size_t scan_temp_bytes(uint32_t n);
 cudaError_t launch_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n, void* tmp,
                                   uint32_t* d_total, cudaStream_t s);
 
-// rips_sort.cu: LSD radix sort of 64-bit keys (optionally with uint32 values),
-// over bits [0, key_bits).  Result in *out (may alias one of the two buffers).
+// rips_sort.cu: LSD radix sort of 64-bit keys (optionally with uint32 values)
+// by bits [low_bit, key_bits), stable; up to SMALL_SORT keys without values are
+// sorted by all their bits in one block.  *result_in_alt tells which of the two
+// buffers holds the result.
+constexpr int RS_TILE = 2048;  // keys per block of a radix pass
+constexpr uint32_t SMALL_SORT = 8192;
 size_t sort_temp_bytes(uint32_t n);
 cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt,
-                           uint32_t n, int key_bits, void* tmp, size_t tmp_bytes, bool* result_in_alt,
+                           uint32_t n, int low_bit, int key_bits, void* tmp, size_t tmp_bytes, bool* result_in_alt,
                            cudaStream_t s);
 
 // One dimension of the reduction (rips_dim.cu)

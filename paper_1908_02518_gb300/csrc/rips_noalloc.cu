@@ -47,7 +47,7 @@ constexpr size_t OFF_TILEOFF = OFF_CLOUD + al(sizeof(CloudInfo));
 constexpr size_t OFF_COUNTS = OFF_TILEOFF + al(2 * 4);   // [0] edges, [1] error flags, [2] per-cloud edges
 constexpr size_t OFF_STATS = OFF_COUNTS + al(4 * 4);
 constexpr size_t OFF_SORT = OFF_STATS + al(16 * 8);
-constexpr size_t SORT_TMP_BYTES = ((NA_MAX_EDGES + 4095) / 4096 * 256 + 256) * 4;
+constexpr size_t SORT_TMP_BYTES = ((NA_MAX_EDGES + RS_TILE - 1) / RS_TILE * 256 + 256) * 4;
 constexpr size_t NOALLOC_BYTES = OFF_SORT + al(SORT_TMP_BYTES);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
@@ -155,7 +155,7 @@ extern "C" RIPS_API int rips_h0_barcode_noalloc(const float* d_dist, int64_t n, 
                          (uint32_t)m_cap, s);
   bool alt = false;
   if (e == cudaSuccess && m_cap > 1)
-    e = radix_sort_u64(keys, keys_alt, nullptr, nullptr, (uint32_t)m_cap, 32 + NA_EDGE_BITS, sort_tmp,
+    e = radix_sort_u64(keys, keys_alt, nullptr, nullptr, (uint32_t)m_cap, 0, 32 + NA_EDGE_BITS, sort_tmp,
                        SORT_TMP_BYTES, &alt, s);
   const uint64_t* sorted = alt ? keys_alt : keys;
   if (e == cudaSuccess) {

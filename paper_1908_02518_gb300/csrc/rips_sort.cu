@@ -3,11 +3,19 @@
 // realises "diameter, then index").
 //
 // Radix sort: 8-bit digits, one pass per digit.  Each pass is
-//   (1) tile histograms      hist[digit][tile]   (digit-major),
-//   (2) per-digit scan over tiles plus digit totals,
+//   (1) tile histograms,
+//   (2) for long inputs a per-digit scan over the tiles (for short ones every
+//       scatter block adds up the tiles before its own itself),
 //   (3) stable scatter: every warp ranks its 32-key steps with
 //       __match_any_sync, warps are ordered by a shared-memory prefix, so keys
-//       with equal digits keep their relative order (LSD correctness).
+//       with equal digits keep their relative order (LSD correctness); the
+//       tile is put in digit order in shared memory and written out in runs.
+// Bits below `low_bit` are not sorted: callers whose keys already come in the
+// order of those bits save their passes.  Bound by L2 and HBM traffic for long
+// inputs (3 x 8 bytes a key and pass: 8.4 million keys 95 us a pass, 140 us when
+// keys were scattered straight from registers after being ranked twice) and by
+// launches for short ones (11000 keys: 0.06 ms in 4 or 5 passes of two launches,
+// 0.14 in 7 of three).  Tiles of 2048 keys give 50 blocks at 100000 keys.
 
 #include <atomic>
 
@@ -99,6 +107,36 @@ __global__ void scan_apply_kernel(const uint32_t* __restrict__ in, uint32_t* __r
     e += v[i];
   }
 }
+
+// the whole scan by one block, tile after tile (in place allowed: a tile is read before it is written)
+__global__ void __launch_bounds__(SCAN_THREADS) scan_one_kernel(const uint32_t* in, uint32_t* out, uint32_t n,
+                                                                uint32_t* __restrict__ total) {
+  __shared__ uint32_t sm[33];
+  uint32_t carry = 0;
+  for (uint32_t base = 0; base < n; base += SCAN_TILE) {
+    uint32_t v[SCAN_ITEMS];
+    uint32_t s = 0;
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+      const uint32_t idx = base + threadIdx.x * SCAN_ITEMS + i;
+      v[i] = idx < n ? in[idx] : 0;
+      s += v[i];
+    }
+    uint32_t tot;
+    uint32_t e = carry + block_excl_scan(s, sm, &tot);
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+      const uint32_t idx = base + threadIdx.x * SCAN_ITEMS + i;
+      if (idx < n) out[idx] = e;
+      e += v[i];
+    }
+    carry += tot;
+  }
+  if (threadIdx.x == 0 && total) *total = carry;
+}
+
+// up to this many values one block scans them (one launch, 2 to 7 us) instead of three kernels (3 launches, 7 us)
+constexpr uint32_t SCAN_ONE = 4 * SCAN_TILE;
 }  // namespace
 
 size_t scan_temp_bytes(uint32_t n) {
@@ -111,6 +149,11 @@ cudaError_t launch_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n,
   uint32_t nb = (uint32_t)(((size_t)n + SCAN_TILE - 1) / SCAN_TILE);
   if (nb == 0) nb = 1;
   uint32_t* sums = (uint32_t*)tmp;
+  if (n <= SCAN_ONE) {
+    scan_one_kernel<<<1, SCAN_THREADS, 0, s>>>(in, out, n, d_total);
+    note_launch();
+    return cudaGetLastError();
+  }
   scan_reduce_kernel<<<nb, SCAN_THREADS, 0, s>>>(in, n, sums);
   note_launch();
   scan_sums_kernel<<<1, SCAN_THREADS, 0, s>>>(sums, nb, d_total);
@@ -124,23 +167,27 @@ cudaError_t launch_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n,
 namespace {
 constexpr int RS_THREADS = 256;   // 8 warps
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_STEPS = 16;      // 32-key steps per warp
-constexpr int RS_TILE = RS_WARPS * RS_STEPS * 32;  // 4096 keys per tile
+constexpr int RS_STEPS = RS_TILE / RS_THREADS;  // 32-key steps per warp
 constexpr int RADIX = 256;
+// Up to this many tiles a scatter block adds up the counts of the tiles before
+// its own (64 rows of 1 KB from L2 at most, about 3 us) instead of a scan launch
+// between (about 3 us at any size).
+constexpr uint32_t RS_DIRECT_TILES = 64;
 
-__global__ void __launch_bounds__(RS_THREADS) rs_hist_kernel(const uint64_t* __restrict__ keys, uint32_t n,
-                                                             int shift, uint32_t* __restrict__ hist,
-                                                             uint32_t tiles) {
+__global__ void __launch_bounds__(RS_THREADS) rs_hist_kernel(const uint64_t* __restrict__ keys, uint32_t n, int shift,
+                                                             uint32_t* __restrict__ hist, uint32_t dstride,
+                                                             uint32_t tstride) {
   __shared__ uint32_t h[RADIX];
-  for (int i = threadIdx.x; i < RADIX; i += RS_THREADS) h[i] = 0;
+  h[threadIdx.x] = 0;
   __syncthreads();
-  size_t base = (size_t)blockIdx.x * RS_TILE;
-  for (int i = threadIdx.x; i < RS_TILE; i += RS_THREADS) {
-    size_t idx = base + i;
+  const size_t base = (size_t)blockIdx.x * RS_TILE;
+#pragma unroll
+  for (int i = 0; i < RS_STEPS; ++i) {
+    const size_t idx = base + i * RS_THREADS + threadIdx.x;
     if (idx < n) atomicAdd(&h[(uint32_t)(keys[idx] >> shift) & 0xFFu], 1u);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < RADIX; i += RS_THREADS) hist[(size_t)i * tiles + blockIdx.x] = h[i];
+  hist[(size_t)threadIdx.x * dstride + (size_t)blockIdx.x * tstride] = h[threadIdx.x];
 }
 
 // one block per digit: exclusive scan of hist[digit][0..tiles) and digit total
@@ -159,74 +206,87 @@ __global__ void rs_tile_scan_kernel(uint32_t* __restrict__ hist, uint32_t tiles,
   if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
-template <bool HAS_VALS>
+// DIRECT: hist is [tile][digit] counts; else [digit][tile] prefixes with the digits' totals
+template <bool HAS_VALS, bool DIRECT>
 __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(
     const uint64_t* __restrict__ keys, uint64_t* __restrict__ keys_out, const uint32_t* __restrict__ vals,
     uint32_t* __restrict__ vals_out, uint32_t n, int shift, const uint32_t* __restrict__ hist, uint32_t tiles,
     const uint32_t* __restrict__ totals) {
-  __shared__ uint32_t digit_base[RADIX];          // global start of each digit
-  __shared__ uint32_t warp_cnt[RS_WARPS][RADIX];  // per-warp digit counts -> running positions
+  __shared__ uint64_t stage[RS_TILE];
+  __shared__ uint32_t stage_v[HAS_VALS ? RS_TILE : 1];
+  __shared__ uint32_t delta[RADIX];               // output position minus position in the tile, per digit
+  __shared__ uint32_t warp_cnt[RS_WARPS][RADIX];  // per-warp digit counts -> the warp's first position in the tile
   __shared__ uint32_t sm[33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, dg = threadIdx.x;  // thread dg owns digit dg
   const unsigned lt_mask = (1u << lane) - 1u;
+  const size_t tile0 = (size_t)blockIdx.x * RS_TILE, base = tile0 + (size_t)warp * RS_STEPS * 32;
 
-  // digit starts: exclusive scan of the digit totals
-  {
-    uint32_t v = threadIdx.x < RADIX ? totals[threadIdx.x] : 0;
-    uint32_t tot;
-    uint32_t e = block_excl_scan(v, sm, &tot);
-    if (threadIdx.x < RADIX) digit_base[threadIdx.x] = e + hist[(size_t)threadIdx.x * tiles + blockIdx.x];
+  uint64_t k[RS_STEPS];
+  uint32_t v[HAS_VALS ? RS_STEPS : 1], pos[RS_STEPS];
+#pragma unroll
+  for (int st = 0; st < RS_STEPS; ++st) {
+    const size_t idx = base + st * 32 + lane;
+    k[st] = idx < n ? keys[idx] : ~0ull;
+    if (HAS_VALS) v[st] = idx < n ? vals[idx] : 0u;
   }
   for (int i = threadIdx.x; i < RS_WARPS * RADIX; i += RS_THREADS) (&warp_cnt[0][0])[i] = 0;
-  __syncthreads();
+  // this tile's first output position of every digit
+  uint32_t mine = 0, all = 0, tot;
+  if (DIRECT) {
+    for (uint32_t t = 0; t < tiles; ++t) {
+      const uint32_t c = hist[(size_t)t * RADIX + dg];
+      if (t == blockIdx.x) mine = all;
+      all += c;
+    }
+  } else {
+    mine = hist[(size_t)dg * tiles + blockIdx.x];
+    all = totals[dg];
+  }
+  mine += block_excl_scan(all, sm, &tot);  // its barriers also order the clearing of the counts
 
-  const size_t base = (size_t)blockIdx.x * RS_TILE + (size_t)warp * RS_STEPS * 32;
-  uint64_t k[RS_STEPS];
+  // rank of every key among its warp's keys of the same digit
 #pragma unroll
   for (int st = 0; st < RS_STEPS; ++st) {
-    size_t idx = base + st * 32 + lane;
-    k[st] = idx < n ? keys[idx] : ~0ull;
-  }
-  // (A) per-warp digit counts
-#pragma unroll
-  for (int st = 0; st < RS_STEPS; ++st) {
-    size_t idx = base + st * 32 + lane;
-    bool valid = idx < n;
-    uint32_t dg = (uint32_t)(k[st] >> shift) & 0xFFu;
-    unsigned act = __ballot_sync(0xffffffffu, valid);
+    const bool valid = base + st * 32 + lane < n;
+    const uint32_t d = (uint32_t)(k[st] >> shift) & 0xFFu;
+    const unsigned act = __ballot_sync(0xffffffffu, valid);
     if (valid) {
-      unsigned peers = __match_any_sync(act, dg);
-      if ((peers & lt_mask) == 0) warp_cnt[warp][dg] += __popc(peers);
-    }
-    __syncwarp();
-  }
-  __syncthreads();
-  // (B) exclusive prefix across warps, per digit
-  for (int dg = threadIdx.x; dg < RADIX; dg += RS_THREADS) {
-    uint32_t run = digit_base[dg];
-    for (int w = 0; w < RS_WARPS; ++w) {
-      uint32_t c = warp_cnt[w][dg];
-      warp_cnt[w][dg] = run;
-      run += c;
-    }
-  }
-  __syncthreads();
-  // (C) stable ranks and scatter
-#pragma unroll
-  for (int st = 0; st < RS_STEPS; ++st) {
-    size_t idx = base + st * 32 + lane;
-    bool valid = idx < n;
-    uint32_t dg = (uint32_t)(k[st] >> shift) & 0xFFu;
-    unsigned act = __ballot_sync(0xffffffffu, valid);
-    if (valid) {
-      unsigned peers = __match_any_sync(act, dg);
-      uint32_t pos = warp_cnt[warp][dg] + __popc(peers & lt_mask);
-      keys_out[pos] = k[st];
-      if (HAS_VALS) vals_out[pos] = vals[idx];
+      const unsigned peers = __match_any_sync(act, d);
+      pos[st] = warp_cnt[warp][d] + __popc(peers & lt_mask);
       __syncwarp(act);
-      if ((peers & lt_mask) == 0) warp_cnt[warp][dg] += __popc(peers);
+      if ((peers & lt_mask) == 0) warp_cnt[warp][d] += __popc(peers);
     }
     __syncwarp();
+  }
+  __syncthreads();
+  // digit by digit and warp by warp: positions in the tile
+  uint32_t cnt = 0;
+#pragma unroll
+  for (int w = 0; w < RS_WARPS; ++w) cnt += warp_cnt[w][dg];
+  uint32_t run = block_excl_scan(cnt, sm, &tot);
+  delta[dg] = mine - run;
+#pragma unroll
+  for (int w = 0; w < RS_WARPS; ++w) {
+    const uint32_t c = warp_cnt[w][dg];
+    warp_cnt[w][dg] = run;
+    run += c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int st = 0; st < RS_STEPS; ++st) {
+    if (base + st * 32 + lane < n) {
+      const uint32_t at = warp_cnt[warp][(uint32_t)(k[st] >> shift) & 0xFFu] + pos[st];
+      stage[at] = k[st];
+      if (HAS_VALS) stage_v[at] = v[st];
+    }
+  }
+  __syncthreads();
+  const uint32_t valid_n = (uint32_t)(n - tile0 < RS_TILE ? n - tile0 : RS_TILE);
+  for (uint32_t i = threadIdx.x; i < valid_n; i += RS_THREADS) {
+    const uint64_t key = stage[i];
+    const uint32_t out = delta[(uint32_t)(key >> shift) & 0xFFu] + i;
+    keys_out[out] = key;
+    if (HAS_VALS) vals_out[out] = stage_v[i];
   }
 }
 }  // namespace
@@ -237,54 +297,90 @@ size_t sort_temp_bytes(uint32_t n) {
   return (tiles * RADIX + RADIX) * sizeof(uint32_t);
 }
 
-// Up to SMALL_SORT keys without values: one block sorts them in shared memory
-// with a bitonic network, in one launch instead of three per radix digit.
-// Without values the order of equal keys does not show, so the result is the
-// radix sort's.
-constexpr uint32_t SMALL_SORT = 8192;
+// Up to SMALL_SORT keys without values: one block sorts them with a bitonic
+// network, in one launch instead of two or three per radix digit.  Without
+// values the order of equal keys does not show, so the result is the radix
+// sort's.  A thread holds 8 consecutive keys: strides below 8 are exchanged in
+// its registers, strides below 256 by shuffles, and only longer ones (15 of the
+// 91 steps of 8192 keys) go through shared memory, in two buffers taken in turn
+// so that a step has one barrier.  4950 keys: 20 us; 50 with every step in
+// shared memory.
+constexpr int SMALL_KEYS = 8;
 
-__global__ void __launch_bounds__(1024) sort_small_kernel(uint64_t* __restrict__ keys, uint32_t n, uint32_t n2) {
-  extern __shared__ uint64_t k[];
-  for (uint32_t i = threadIdx.x; i < n2; i += blockDim.x) k[i] = i < n ? keys[i] : ~0ull;
-  __syncthreads();
+__global__ void __launch_bounds__(SMALL_SORT / SMALL_KEYS) sort_small_kernel(uint64_t* __restrict__ keys, uint32_t n) {
+  extern __shared__ uint64_t sbuf[];
+  const uint32_t T = blockDim.x, t = threadIdx.x, n2 = T * SMALL_KEYS;
+  uint64_t k[SMALL_KEYS];
+#pragma unroll
+  for (int e = 0; e < SMALL_KEYS; ++e) {  // any assignment will do before the first step: the coalesced one
+    const uint32_t i = e * T + t;
+    k[e] = i < n ? keys[i] : ~0ull;
+  }
+  uint64_t* buf = sbuf;
   for (uint32_t size = 2; size <= n2; size <<= 1) {
-    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      for (uint32_t i = threadIdx.x; i < n2; i += blockDim.x) {
-        const uint32_t l = i ^ stride;
-        if (l > i) {
-          const uint64_t a = k[i], b = k[l];
-          if ((a > b) == ((i & size) == 0)) {
-            k[i] = b;
-            k[l] = a;
+    for (uint32_t stride = size >> 1; stride >= SMALL_KEYS; stride >>= 1) {
+      const uint32_t far = stride / SMALL_KEYS;  // distance in threads; size > stride: one direction a thread
+      const bool low = (((t * SMALL_KEYS) & stride) == 0) == (((t * SMALL_KEYS) & size) == 0);
+      if (far < 32) {
+#pragma unroll
+        for (int e = 0; e < SMALL_KEYS; ++e) {
+          const uint64_t o = __shfl_xor_sync(0xffffffffu, k[e], far);
+          k[e] = (o < k[e]) == low ? o : k[e];
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < SMALL_KEYS; ++e) buf[e * T + t] = k[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < SMALL_KEYS; ++e) {
+          const uint64_t o = buf[e * T + (t ^ far)];
+          k[e] = (o < k[e]) == low ? o : k[e];
+        }
+        buf = buf == sbuf ? sbuf + n2 : sbuf;
+      }
+    }
+#pragma unroll
+    for (int stride = SMALL_KEYS / 2; stride > 0; stride >>= 1) {
+      if ((uint32_t)stride < size) {
+#pragma unroll
+        for (int e = 0; e < SMALL_KEYS; ++e) {
+          if ((e & stride) == 0) {
+            const uint64_t x = k[e], y = k[e | stride];
+            const bool swap = (x > y) == (((t * SMALL_KEYS + e) & size) == 0);
+            k[e] = swap ? y : x;
+            k[e | stride] = swap ? x : y;
           }
         }
       }
-      __syncthreads();
     }
   }
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) keys[i] = k[i];
+#pragma unroll
+  for (int e = 0; e < SMALL_KEYS; ++e) {
+    const uint32_t i = t * SMALL_KEYS + e;
+    if (i < n) keys[i] = k[e];
+  }
 }
 
 cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint32_t n,
-                           int key_bits, void* tmp, size_t tmp_bytes, bool* result_in_alt, cudaStream_t s) {
+                           int low_bit, int key_bits, void* tmp, size_t tmp_bytes, bool* result_in_alt, cudaStream_t s) {
   *result_in_alt = false;
-  if (n <= 1 || key_bits <= 0) return cudaSuccess;
+  if (n <= 1 || key_bits <= low_bit) return cudaSuccess;
   if (!vals && n <= SMALL_SORT) {
-    uint32_t n2 = 2;
-    while (n2 < n) n2 <<= 1;
-    const size_t smem = (size_t)n2 * 8;
+    uint32_t threads = 32;
+    while (threads * SMALL_KEYS < n) threads <<= 1;
+    const size_t smem = threads > 32 ? (size_t)threads * SMALL_KEYS * 16 : 0;
     if (smem > 48 * 1024) {
       static std::atomic<bool> opted[64];  // once per device (any thread)
       int dev = 0;
       cudaError_t e = cudaGetDevice(&dev);
       if (e != cudaSuccess) return e;
       if (dev < 0 || dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SMALL_SORT * 8));
+        e = cudaFuncSetAttribute(sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SMALL_SORT * 16));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) opted[dev].store(true, std::memory_order_release);
       }
     }
-    sort_small_kernel<<<1, 1024, smem, s>>>(keys, n, n2);
+    sort_small_kernel<<<1, threads, smem, s>>>(keys, n);
     note_launch();
     return cudaGetLastError();
   }
@@ -297,16 +393,25 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, u
   uint32_t* vin = vals;
   uint32_t* vout = vals_alt;
   bool alt = false;
-  for (int shift = 0; shift < key_bits; shift += 8) {
-    rs_hist_kernel<<<tiles, RS_THREADS, 0, s>>>(kin, n, shift, hist, tiles);
+  const bool direct = tiles <= RS_DIRECT_TILES;
+  for (int shift = low_bit; shift < key_bits; shift += 8) {
+    rs_hist_kernel<<<tiles, RS_THREADS, 0, s>>>(kin, n, shift, hist, direct ? 1 : tiles, direct ? RADIX : 1);
     note_launch();
-    rs_tile_scan_kernel<<<RADIX, 256, 0, s>>>(hist, tiles, totals);
-    note_launch();
-    if (vals)
-      rs_scatter_kernel<true><<<tiles, RS_THREADS, 0, s>>>(kin, kout, vin, vout, n, shift, hist, tiles, totals);
-    else
-      rs_scatter_kernel<false><<<tiles, RS_THREADS, 0, s>>>(kin, kout, nullptr, nullptr, n, shift, hist, tiles,
-                                                            totals);
+    if (direct) {
+      if (vals)
+        rs_scatter_kernel<true, true><<<tiles, RS_THREADS, 0, s>>>(kin, kout, vin, vout, n, shift, hist, tiles, totals);
+      else
+        rs_scatter_kernel<false, true><<<tiles, RS_THREADS, 0, s>>>(kin, kout, nullptr, nullptr, n, shift, hist, tiles,
+                                                                    totals);
+    } else {
+      rs_tile_scan_kernel<<<RADIX, 256, 0, s>>>(hist, tiles, totals);
+      note_launch();
+      if (vals)
+        rs_scatter_kernel<true, false><<<tiles, RS_THREADS, 0, s>>>(kin, kout, vin, vout, n, shift, hist, tiles, totals);
+      else
+        rs_scatter_kernel<false, false><<<tiles, RS_THREADS, 0, s>>>(kin, kout, nullptr, nullptr, n, shift, hist, tiles,
+                                                                     totals);
+    }
     note_launch();
     uint64_t* t = kin;
     kin = kout;
