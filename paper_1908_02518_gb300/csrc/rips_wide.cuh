@@ -22,12 +22,16 @@
 // the rows beyond are in the table only.  A round extends the front from the mid
 // list, up to a key sampled so that about K rows join it, looks its rows over,
 // writes the live owned ones into a work list, and then adds their owners, one
-// warp a row.  The mid list is refilled by a scan of the table.  K is a third of the additions made so far (8 at
-// first), so a chain of A additions takes on the order of log2(A) rounds and the
-// additions wasted on rows past its pivot are a share of A.  A window whose rows
-// multiply is cut back to K.  (K counts rows that have an owner: the window is
-// extended by the share of such rows the last time.)  Rows behind the window are settled; a table that
-// fills up is rebuilt from its live rows.
+// warp a row.  The mid list is refilled by a scan of the table.  K grows with the
+// additions made so far, so a chain of A additions takes on the order of log2(A)
+// rounds and the additions wasted on rows past its pivot are a share of A: a
+// third of them and at least 8 for a block, since other columns wait for it; for
+// a team as many as made, between 32 and 512, and half as many beyond, since half
+// of the chip waits for a team and a round costs it a barrier over blocks more.  A
+// window whose rows multiply is cut back to K.  (K counts rows that have an
+// owner: the window is extended by the share of such rows the last time.)  Rows
+// behind the window are settled; a table that fills up is rebuilt from its live
+// rows.
 //
 // What bounds it: memory latency.  A section is a handful of dependent round
 // trips (a row's slot, value and owner: 5 to 7 us; a coboundary's neighbours,
@@ -51,6 +55,13 @@ constexpr uint32_t SORT_RUN = 1024;  // stored runs up to this length are sorted
 constexpr uint64_t OWN_TABLE = 13, OWN_NONE = 14, OWN_UNKNOWN = 15;  // OWN_TABLE | (ordinal << 4)
 
 constexpr uint32_t WIDE_K0 = 8;         // rows of the first window
+// Rows of a team's window: as many as additions made, between these, and half as many beyond.  Measured against a third
+// of them, at least 8, for teams too: torus of 1,000 points to H2 3.58 -> 2.82 ms, 1,500 points of a Clifford torus
+// 4.76 -> 3.77, edge list of 4,999 points 13.8 -> 11.7, 2,048 rotations 18.1 -> 16.1, 24-cloud plan 3.22 -> 2.88,
+// 32 clouds 24.9 -> 24.0.  Windows this wide in single blocks cost more than they save while blocks are short (32
+// clouds 24.9 -> 25.3 to 28.6, 100 points 0.75 -> 0.80 to 0.85), all additions past 512 too (3-sphere of 144 points
+// over Z/3 15.7 -> 16.6).
+constexpr uint32_t WIDE_TEAM_K0 = 32, WIDE_TEAM_K1 = 512;
 constexpr uint32_t WIDE_SAMPLES = 128;   // keys sampled to place a bound, one a thread
 constexpr uint32_t TEAM_MIN_ROWS = 1024;  // stored rows from which a column starts with a team
 constexpr uint32_t TEAM_MIN_STEPS = 32;  // additions a block makes before it gives its column to a team
@@ -1027,7 +1038,9 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
   uint32_t last = 0;        // rows added last round
   float share = 1.0f;       // of k, to extend the window by
   for (;;) {
-    const uint32_t k = min(max(w.step / 3, WIDE_K0), kmax);  // rows with an owner wanted in the window
+    const uint32_t goal = t.size > 1 ? max(w.step / 2, min(max(w.step, WIDE_TEAM_K0), WIDE_TEAM_K1))
+                                     : max(w.step / 3, WIDE_K0);
+    const uint32_t k = min(goal, kmax);  // rows with an owner wanted in the window
     const unsigned long long want = max(1ull, min((unsigned long long)((float)k * share) * w.dil, rows));
     bool extend = false;
     uint64_t b = w.bound;
