@@ -61,16 +61,46 @@ namespace rips {
 
 // ====================================================================== enumeration
 
+// A warp takes a (d-1)-simplex and 32 candidates of its shortest neighbour list at
+// a time, and gathers what it finds in shared memory, up to ENUM_BUF simplices
+// that take their place in the list with one atomic.  All warps share that one
+// counter: an atomic for every 32 candidates bound the kernel (3-sphere of 144
+// points, 13.9 million simplices: 0.50 -> 0.26 ms; 2,048 rotations, 2.2 million
+// triangles: 0.147 -> 0.071; 4,096, 17.5 million: 0.96 -> 0.37).
+// D = d keeps the vertices in registers and issues a candidate's rank lookups
+// together; 0: any d.
+constexpr int ENUM_BUF = 128;
+
+template <int D>
 __global__ void __launch_bounds__(256) enumerate_kernel(DimArgs a, const uint64_t* __restrict__ pidx,
                                                         const uint32_t* __restrict__ prank, uint32_t np, int pbits,
                                                         uint64_t* __restrict__ out_idx, uint32_t* __restrict__ out_rank,
                                                         unsigned long long* __restrict__ count,
                                                         unsigned long long cap) {
   extern __shared__ uint64_t smem[];
+  __shared__ uint64_t buf_idx[WARPS_PER_BLOCK][ENUM_BUF];
+  __shared__ uint32_t buf_rank[WARPS_PER_BLOCK][ENUM_BUF];
   Binom B = stage_binom(a, smem);
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const int d = a.d;  // new simplices are d-simplices, made from (d-1)-simplices
+  const int d = D ? D : a.d;  // new simplices are d-simplices, made from (d-1)-simplices
+  constexpr int NV = D ? D : MAX_DIM + 2;
+  uint64_t* const bi = buf_idx[threadIdx.x >> 5];
+  uint32_t* const br = buf_rank[threadIdx.x >> 5];
+  int held = 0;  // simplices in the warp's buffer
+  auto flush = [&]() {
+    __syncwarp();
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(count, (unsigned long long)held);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (int i = lane; i < held; i += 32)
+      if (base + i < cap) {
+        out_idx[base + i] = bi[i];
+        out_rank[base + i] = br[i];
+      }
+    __syncwarp();
+    held = 0;
+  };
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < np; s += warps) {
     const uint64_t g = pidx[s];
@@ -78,42 +108,63 @@ __global__ void __launch_bounds__(256) enumerate_kernel(DimArgs a, const uint64_
     const uint64_t local = g & low_mask(pbits);
     const CV cv = cloud_view(a, cl);
     const uint64_t chi = a.col_bits >= 64 ? 0ull : ((uint64_t)cl << a.col_bits);
-    int v[MAX_DIM + 2];
-    decode(B, cv.n, local, d - 1, v);
+    int v[NV];
+    int hi = cv.n - 1;
+    uint64_t N = local;
+    uint32_t beg = 0, end = ~0u;  // the shortest list of a vertex
+#pragma unroll
+    for (int l = 0; l < NV; ++l)
+      if (l < d) {
+        const int k = d - l;
+        v[l] = k == 1 ? (int)N : max_vertex(B, k, hi, N);
+        N -= k == 1 ? N : B(v[l], k);
+        hi = v[l] - 1;
+        const uint32_t o0 = cv.off[v[l]], o1 = cv.off[v[l] + 1];
+        if (o1 - o0 < end - beg) {
+          beg = o0;
+          end = o1;
+        }
+      }
     const uint32_t r0 = prank[s];
     const int top = v[0];
-    const int av = v[min_degree_vertex(cv, v, d)];
-    const uint32_t beg = cv.off[av], end = cv.off[av + 1];
     for (uint32_t q0 = beg; q0 < end; q0 += 32) {
       const uint32_t q = q0 + lane;
-      int j = q < end ? (int)cv.nbr[q] : -1;
+      const int j = q < end ? (int)cv.nbr[q] : -1;
       bool ok = j > top;
       uint32_t r = r0;
-      if (ok)
-        for (int l = 0; l < d; ++l) {
-          uint32_t x = rank_of(cv, v[l], j);
-          if (x == RANK_INF) {
-            ok = false;
-            break;
+      if (ok) {
+        if (D && cv.R) {
+#pragma unroll
+          for (int l = 0; l < NV; ++l) r = max(r, cv.R[(size_t)v[l] * cv.n + j]);
+          ok = r != RANK_INF;
+        } else {
+          for (int l = 0; l < d; ++l) {
+            uint32_t x = RANK_INF;
+#pragma unroll
+            for (int y = 0; y < NV; ++y)
+              if (y == l) x = rank_of(cv, v[y], j);
+            if (x == RANK_INF) {
+              ok = false;
+              break;
+            }
+            r = max(r, x);
           }
-          r = max(r, x);
         }
-      unsigned m = __ballot_sync(0xffffffffu, ok);
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, ok);
       if (m) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(count, (unsigned long long)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
+        if (held + __popc(m) > ENUM_BUF) flush();
         if (ok) {
-          unsigned long long pos = base + __popc(m & lt);
-          if (pos < cap) {
-            out_idx[pos] = chi | (local + B(j, d + 1));
-            out_rank[pos] = r;
-          }
+          const int at = held + __popc(m & lt);
+          bi[at] = chi | (local + B(j, d + 1));
+          br[at] = r;
         }
+        held += __popc(m);
       }
       if (!__all_sync(0xffffffffu, j > top)) break;  // the list went below the top vertex
     }
   }
+  if (held) flush();
 }
 
 // edges (sorted) -> simplex list of dimension 1
@@ -462,12 +513,15 @@ cudaError_t launch_enumerate(const DimArgs& a, const uint64_t* pidx, const uint3
                              unsigned long long cap, cudaStream_t st) {
   if (np == 0) return cudaSuccess;
   size_t sm = binom_smem(a);
-  cudaError_t e = prepare((const void*)enumerate_kernel, sm);
+  const void* kernel = a.d == 2 ? (const void*)enumerate_kernel<2>
+                       : a.d == 3 ? (const void*)enumerate_kernel<3> : (const void*)enumerate_kernel<0>;
+  cudaError_t e = prepare(kernel, sm);
   if (e != cudaSuccess) return e;
-  enumerate_kernel<<<grid_for_warps(np, a.scan_blocks_per_sm), 256, sm, st>>>(a, pidx, prank, np, prev_col_bits, out_idx, out_rank, count,
-                                                        cap);
+  DimArgs aa = a;
+  void* args[] = {&aa, &pidx, &prank, &np, &prev_col_bits, &out_idx, &out_rank, &count, &cap};
+  e = cudaLaunchKernel(kernel, dim3(grid_for_warps(np, a.scan_blocks_per_sm)), dim3(256), args, sm, st);
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_edges_to_simplices(const uint64_t* keys, const uint32_t* erank, uint32_t m, int edge_bits,
