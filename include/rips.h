@@ -397,9 +397,9 @@ RIPS_API uint32_t rips_get_options(void);
  * rips_batch_plan_result waits for the stream and returns the last run's bars
  * and statistics as a result (for the accessors and rips_barcodes_backward).
  * The reduction's arena is fixed too: arena_entries entries of 12 bytes (0:
- * 384 per edge, within 40 % of the free device memory; the arena keeps every
- * intermediate run of a reduction, 150 to 250 entries per edge on the 256-cloud
- * mix of circles, tori and cubes); a run that needs more
+ * 384 per edge, within 40 % of the free device memory) for stored columns, and
+ * beside them, as far as the 40 % leave room, the tables and lists of the columns
+ * under way (at most 1664 per edge); a run that needs more
  * reports RIPS_ERR_OOM from rips_batch_plan_result.  A plan is used by one
  * stream at a time. */
 typedef struct rips_batch_plan rips_batch_plan_t;

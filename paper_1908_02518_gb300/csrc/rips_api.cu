@@ -1300,18 +1300,25 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   a.opts = 0;  // batch plans always take both shortcuts
   pl.tcap = pow2_at_least(2ull * pl.e_cap + 16);
   pl.acap = pow2_at_least(2ull * pl.e_cap + 16);
-  if (arena_entries) {
-    pl.arena = (size_t)arena_entries;
-  } else {  // every merge and generated coboundary takes new arena space: 384 entries per edge, within 40 % of free memory
+  pl.slice = 32;
+  while (pl.slice < (uint32_t)pl.n_max + 1) pl.slice <<= 1;
+  pl.blocks = reduction_blocks(a, (uint32_t)pl.e_cap);
+  if (pl.blocks < 1) return RIPS_ERR_CUDA;
+  {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
       cudaGetLastError();
       free_b = (size_t)16 << 30;
     }
-    pl.arena = std::max<size_t>(std::min<size_t>(384 * (size_t)pl.e_cap, free_b / 12 * 2 / 5), (size_t)1 << 22);
+    const size_t fit = free_b / 12 * 2 / 5;
+    // the caller's entries, or 384 per edge within 40 % of free memory, for stored columns and generated coboundaries
+    pl.arena = arena_entries ? (size_t)arena_entries
+                             : std::max<size_t>(std::min<size_t>(384 * (size_t)pl.e_cap, fit), (size_t)1 << 22);
+    // and, as far as that leaves room within the 40 %, the tables and lists of the columns under way: a block's are a
+    // few tens of its first ones' size (96 entries a slot of a coboundary) by the time its columns have grown
+    const size_t tables = std::min<size_t>(1664 * (size_t)pl.e_cap, (size_t)3072 * pl.slice * (size_t)pl.blocks);
+    if (pl.arena < fit) pl.arena += std::min(tables, fit - pl.arena);
   }
-  pl.slice = 32;
-  while (pl.slice < (uint32_t)pl.n_max + 1) pl.slice <<= 1;
   Workspace& w = pl.w;
   const uint64_t E = pl.e_cap, N = pl.N;
   const size_t SPCB = (size_t)batch * PLAN_SPC * 8;
@@ -1374,8 +1381,6 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   a.amap = P<uint64_t>(w.amk[0]);
   a.amap_mask = pl.acap - 1;
   a.vbits = packed_vertex_bits(pl.n_max, 1);
-  pl.blocks = reduction_blocks(a, (uint32_t)E);
-  if (pl.blocks < 1) return RIPS_ERR_CUDA;
   CR(ensure(w.wide, wide_ctx_bytes(pl.blocks)));
   return RIPS_OK;
 }
