@@ -345,15 +345,29 @@ __device__ float distance_rule(const float* __restrict__ x, const float* __restr
   return __double2float_rn(__dsqrt_rn(acc));
 }
 
-// The same value from FP32 arithmetic, which this GPU does 60 times as fast: the
-// sum is carried as an unevaluated pair of FP32 numbers (error-free differences,
-// squares and sums: Knuth, "The Art of Computer Programming" 2, 4.2.2; Dekker,
-// "A floating-point technique for extending the available precision", 1971), good
-// to about 2^-45 of it; the correction of the rounded root tells which FP32 number
-// is nearest.  Where the root lies too near the middle of two FP32 numbers for
-// that (one pair in 2^15 or fewer), at a power of two, or where the sum leaves
-// the range in which the error terms are exact, `settled` is false and the rule
-// itself is evaluated: the result is the rule's bit for bit.
+// The same value from FP32 arithmetic, which this GPU does 60 times as fast: sums
+// are carried as unevaluated pairs of FP32 numbers (error-free differences, squares
+// and sums: Knuth, "The Art of Computer Programming" 2, 4.2.2; Dekker, "A
+// floating-point technique for extending the available precision", 1971), a pair
+// for DIST_K coordinates at a time, joined into the pair of the whole; the
+// correction of the rounded root tells which FP32 number is nearest.  Where the
+// root lies too near the middle of two FP32 numbers for that (see dist_margin), at
+// a power of two, or where the sum leaves the range in which the error terms are
+// exact, `settled` is false and the rule itself is evaluated: the result is the
+// rule's bit for bit, however many coordinates there are.
+//
+// Error bound, with u = 2^-24, p a coordinate's square, C the sum of a chunk of j
+// coordinates and H the whole.  In add, s + e, s^2 - p and t + r are exact; q is off
+// by 4 u^2 p (its rounding, |q| <= 3 u p, and e^2 <= u^2 p), r + q is rounded to
+// u (u C + 3 u p), and |lo| grows by as much as that over u, to (j + 4) u C, whose
+// rounding costs u times as much: a chunk is off by at most (21 j + 7) u^2 C, all
+// chunks together by (21 min(k, 16) + 7) u^2 H.  join leaves |lo| <= u H and rounds
+// twice, 3 u^2 H + 40 u^2 C.  The sum is thus off by at most (21 k + 7) u^2 H in one
+// chunk and (k / 5 + 386) u^2 H in more, and the root, whose last place is at least
+// u of it, by half as many u of that place; the correction adds less than 3 u, and
+// float64's own roundings (0.75 k + 1) 2^-29.  (In one pair from end to end the
+// error grows with the square of k: from 169 equal differences on, roots came out
+// one unit off.)
 struct PairSum {
   float hi = 0.0f, lo = 0.0f;
   __device__ __forceinline__ void add(float a, float b) {
@@ -366,7 +380,15 @@ struct PairSum {
     hi = t;
     lo = __fadd_rn(lo, __fadd_rn(r, q));
   }
-  // the distance, given margin = 2^-17 + k 2^-23 (in units of the root's last place: four times the error bound)
+  // the sum of other coordinates
+  __device__ __forceinline__ void join(const PairSum& o) {
+    const float t = __fadd_rn(hi, o.hi), y = __fsub_rn(t, hi);
+    const float r = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, y)), __fsub_rn(o.hi, y));  // hi + o.hi = t + r
+    const float l = __fadd_rn(lo, __fadd_rn(r, o.lo));
+    hi = __fadd_rn(t, l);
+    lo = __fsub_rn(l, __fsub_rn(hi, t));  // exact: |l| < t
+  }
+  // the distance, given the margin of dist_margin
   __device__ __forceinline__ float root(float margin, bool* settled) const {
     const float h = __fadd_rn(hi, lo), l = __fsub_rn(lo, __fsub_rn(h, hi));
     const float y = __fsqrt_rn(h);
@@ -385,12 +407,23 @@ struct PairSum {
 // coordinates 16 at a time through shared memory.  256 threads; pairs outside the
 // cloud have ok = false.
 constexpr int DIST_K = 16;
+static_assert(DIST_K == 16, "the bound of PairSum");
+
+// How near the middle of two FP32 numbers a root is left to the rule, in units of
+// its last place: against PairSum's bound, (128 + 16 k) u for (10.5 k + 8) u in one
+// chunk and (384 + k / 4) u for (k / 8 + 197) u in more.  One random pair in 30,000
+// is left at k = 9, one in 13,000 at 1,000.
+__device__ __forceinline__ float dist_margin(int k) {
+  return 0x1p-24f * (128.0f + 16.0f * (float)min(k, DIST_K) + 0.25f * (float)k);
+}
+
 template <class F>
 __device__ __forceinline__ void distance_tile(const float* __restrict__ x, int n, int k, int i0, int j0, F f) {
   __shared__ float xi[32][DIST_K + 1], xj[32][DIST_K + 1];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   PairSum sum[4];
   for (int c0 = 0; c0 < k; c0 += DIST_K) {
+    PairSum part[4];
     const int kc = min(DIST_K, k - c0);
     __syncthreads();
     for (int q = threadIdx.x; q < 32 * DIST_K; q += 256) {
@@ -402,10 +435,15 @@ __device__ __forceinline__ void distance_tile(const float* __restrict__ x, int n
     for (int c = 0; c < kc; ++c) {
       const float b = xj[tx][c];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) sum[r].add(xi[ty + 8 * r][c], b);
+      for (int r = 0; r < 4; ++r) part[r].add(xi[ty + 8 * r][c], b);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (c0 == 0) sum[r] = part[r];
+      else sum[r].join(part[r]);
     }
   }
-  const float margin = 0x1p-17f + (float)k * 0x1p-23f;
+  const float margin = dist_margin(k);
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int i = i0 + ty + 8 * r, j = j0 + tx;
@@ -424,7 +462,8 @@ __device__ __forceinline__ void distance_tile(const float* __restrict__ x, int n
 
 // n x n, both triangles from the tiles of the lower one (a distance is the same
 // both ways, bit for bit): the transposed tile goes out through shared memory.
-// 4,096 points in R^9: 1,672 us in float64 on every ordered pair before.
+// Against float64 on every ordered pair: 4,096 points in R^9 1,671 -> 84 us, 2,048 in
+// R^784 30.4 -> 1.3 ms; with one pair in seven left to the rule (grey levels) 14.5 ms.
 __global__ void __launch_bounds__(256) distance_kernel(const float* __restrict__ pts, int n, int k,
                                                        float* __restrict__ D) {
   __shared__ float tile[32][33];
