@@ -12,6 +12,8 @@
 // a batch at a time, and finds forest and elder rule together by contraction
 // (h0_block_kernel); it stops reading when one component is left.  A larger
 // cloud uses grid-wide Boruvka rounds and then the elder rule over the forest.
+#include <atomic>
+
 #include "rips_internal.cuh"
 
 namespace rips {
@@ -395,10 +397,18 @@ cudaError_t launch_h0_blocks(const CloudInfo* clouds, int nclouds, int n_max, co
   const int threads = n_max <= 256 ? 256 : 1024;
   const uint32_t list_cap = 2u * H0_STEP * (uint32_t)threads;
   const size_t smem = (size_t)12 * (n_max > 0 ? n_max : 1) + (size_t)8 * list_cap;
-  if (smem > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(h0_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-          cudaSuccess)
-    return e;
+  if (smem > 48 * 1024) {
+    // once per device and to the largest size any call needs: calls of other threads are between setting and launching
+    static std::atomic<bool> opted[64];
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
+      constexpr int most = 12 * H0_BLOCK_MAX_N + 8 * 2 * H0_STEP * 1024;
+      if ((e = cudaFuncSetAttribute(h0_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
+        return e;
+      if (dev >= 0 && dev < 64) opted[dev].store(true, std::memory_order_release);
+    }
+  }
   h0_block_kernel<<<nclouds, threads, smem, s>>>(clouds, sorted_keys, edge_bits, in_forest, bars, nbars, bar_cap, stats,
                                                  stats_stride, list_cap);
   note_launch();
