@@ -935,6 +935,10 @@ __device__ bool grid_barrier(unsigned* count, unsigned* gen, const RedState& s, 
 
 }  // namespace
 
+// Entry of the list of suspended columns: the context, and whether the column has
+// made TEAM_LARGE_STEPS additions.
+constexpr unsigned SUSP_LARGE = 0x80000000u;
+
 // The whole reduction of one dimension in one cooperative launch: the first
 // pivots of all columns, then claim / reduce rounds separated by grid
 // barriers, until no column is left to claim or reduce.  The losers of a
@@ -1078,14 +1082,14 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
         }
         // one team left: a grid-wide barrier pays from rounds of thousands of rows on
         uint32_t size = gridDim.x / nteam;
+        // (from the list, which stays as it is in this phase: the team's leader writes the column's state)
         const bool small = nteam == 1 && size > TEAM_SMALL &&
-                           *(volatile uint32_t*)&s.wide[*(volatile unsigned*)&susp_list[(it % 3) * gridDim.x]].st.step <
-                               TEAM_LARGE_STEPS;
+                           !(*(volatile unsigned*)&susp_list[(it % 3) * gridDim.x] & SUSP_LARGE);
         if (small) size = TEAM_SMALL;
         const uint32_t q = blockIdx.x / size;
         team.size = 0;  // none for this block
         if (q < nteam) {
-          c = s.wide + *(volatile unsigned*)&susp_list[(it % 3) * gridDim.x + q];
+          c = s.wide + (*(volatile unsigned*)&susp_list[(it % 3) * gridDim.x + q] & ~SUSP_LARGE);
           if (threadIdx.x == 0) wt = c->st;
           team = Team{(int)size, (int)(blockIdx.x - q * size), &c->sh};
         }
@@ -1108,7 +1112,8 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
           if (st == CH_HEAVY) {
             c->st = w;
             const uint32_t to = queue ? it % 3 : (it + 1) % 3;
-            susp_list[to * gridDim.x + atomicAdd(&susp_cnt[to], 1u)] = (unsigned)(c - s.wide);
+            susp_list[to * gridDim.x + atomicAdd(&susp_cnt[to], 1u)] =
+                (unsigned)(c - s.wide) | (w.step >= TEAM_LARGE_STEPS ? SUSP_LARGE : 0u);
             if (queue) {
               for (int q = 0; q < 3; ++q) wide_clear(&c->sh.c[q]);
               c->sh.bar_count = c->sh.bar_gen = 0;

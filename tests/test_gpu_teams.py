@@ -1,0 +1,36 @@
+"""Teams of blocks (csrc/rips_reduce.cuh), where the blocks of a launch divide
+themselves anew: a column that outlives the others and passes from a block to 64
+of them and, after 4,096 additions, to the whole grid.  Which team a block is in
+follows from lists that stay as they are while the teams run, so every run gives
+the same bars."""
+import math
+
+import pytest
+
+from paper_1908_02518_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+LARGE = 4096  # additions after which a lone column's team grows from 64 blocks to all
+
+# name, distances, dimension, threshold, p, additions of the longest chain at least
+CASES = [("s3_112", lambda: W.distance_matrix(W.sphere_points(112, 1005, 4)), 3, math.inf, 3, LARGE),
+         ("so3_700", lambda: W.distance_matrix(W.so3_points(700, 1005)), 1, math.inf, 2, 32)]
+
+
+def _key(bars):
+    return sorted((int(b["dim"]), float(b["birth"]), float(b["death"]), int(b["birth_simplex"]),
+                   int(b["death_simplex"]) % 2**64) for b in bars)
+
+
+@pytest.mark.parametrize("name,make,dim_max,t,p,chain", CASES, ids=[c[0] for c in CASES])
+def test_columns_that_change_teams(oracle_mod, name, make, dim_max, t, p, chain):
+    import torch
+    import paper_1908_02518_gb300 as rg
+    d = make()
+    want = _key(oracle_mod.barcodes(d, dim_max, t, p).bars)
+    x = torch.from_numpy(d).cuda()
+    for _ in range(10):
+        res = rg.barcodes(x, dim_max, t, p)
+        assert max(s["longest_chain"] for s in res.stats[0]) >= chain
+        assert _key(res.bars) == want
