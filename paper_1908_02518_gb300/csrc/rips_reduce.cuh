@@ -721,13 +721,29 @@ __device__ int chain_warp(const DimArgs& a, const RedState& s, const CV& cv, con
   return CH_DONE;
 }
 
+// The columns that blocks reduce in a round, and whether one of that round (heavy
+// or not) is stored with so many rows that it takes a block long to enter them.
+// Said while columns are listed: a block that looked the rows up in the reduce
+// phase would race with blocks that store reduced columns.
+constexpr uint32_t TEAM_MIN_ROWS = 1024;  // stored rows from which a column starts with a team
+struct HeavyList {
+  uint32_t *count, *list;
+  unsigned* large;
+  __device__ __forceinline__ void put(const RedState& s, uint32_t j) const {
+    list[atomicAdd(count, 1u)] = j;
+    note(s, j);
+  }
+  __device__ __forceinline__ void note(const RedState& s, uint32_t j) const {
+    if (s.r_len[j] > TEAM_MIN_ROWS) *(volatile unsigned*)large = 1u;
+  }
+};
+
 // A warp gives a heavy column up before changing any of its state: the column
 // is flagged and queued for a block in the next round.
-__device__ __forceinline__ void chain_give_up(const RedState& s, int lane, uint32_t j, uint32_t* heavy_count,
-                                              uint32_t* heavy_list) {
+__device__ __forceinline__ void chain_give_up(const RedState& s, int lane, uint32_t j, const HeavyList& heavy) {
   if (lane == 0) {
     s.reduced[j] |= HEAVY;
-    heavy_list[atomicAdd(heavy_count, 1u)] = j;
+    heavy.put(s, j);
   }
 }
 
@@ -772,8 +788,7 @@ __device__ uint64_t first_pivot(const DimArgs& a, const CV& cv, const Binom& B, 
 // to the claim list.
 template <int D>
 __device__ void init_column(const DimArgs& a, const RedState& s, const Binom& B, int lane, const SortTile& tile,
-                            uint32_t j, uint32_t limit, uint32_t* claim_count, uint32_t* heavy_count,
-                            uint32_t* heavy_list) {
+                            uint32_t j, uint32_t limit, uint32_t* claim_count, const HeavyList& heavy) {
   uint64_t idx;
   uint32_t r, cl, coef;
   column_simplex(a, s, j, &idx, &r, &cl);
@@ -792,7 +807,7 @@ __device__ void init_column(const DimArgs& a, const RedState& s, const Binom& B,
       s.piv_key[j] = key;
       s.piv_coef[j] = coef;
     }
-    chain_give_up(s, lane, j, heavy_count, heavy_list);
+    chain_give_up(s, lane, j, heavy);
     return;
   }
   if (st != CH_DONE) {
@@ -804,14 +819,18 @@ __device__ void init_column(const DimArgs& a, const RedState& s, const Binom& B,
 
 // Column j claims its pivot: the smallest ordinal owns it; the loser (j, or the
 // displaced former owner) goes to the reduce list.
-__device__ __forceinline__ void to_reduce(const RedState& s, uint32_t j, uint32_t* reduce_count, uint32_t* heavy_count,
-                                          uint32_t* heavy_list) {
-  if (s.reduced[j] & HEAVY) heavy_list[atomicAdd(heavy_count, 1u)] = j;
-  else s.reduce_list[atomicAdd(reduce_count, 1u)] = j;
+__device__ __forceinline__ void to_reduce(const RedState& s, uint32_t j, uint32_t* reduce_count,
+                                          const HeavyList& heavy) {
+  if (s.reduced[j] & HEAVY) {
+    heavy.put(s, j);
+  } else {
+    s.reduce_list[atomicAdd(reduce_count, 1u)] = j;
+    heavy.note(s, j);
+  }
 }
 
 __device__ void claim_one(const DimArgs& a, const RedState& s, uint32_t j, uint32_t* reduce_count,
-                          uint32_t* heavy_count, uint32_t* heavy_list) {
+                          const HeavyList& heavy) {
   const uint64_t key = s.piv_key[j];
   const uint32_t cl = high_part(s.col_keys[j], a.rank_bits + a.col_bits);
   const int64_t slot = table_insert(s.t_keys, s.t_mask, table_key(a, cl, row_key_idx(a, key)));
@@ -820,8 +839,8 @@ __device__ void claim_one(const DimArgs& a, const RedState& s, uint32_t j, uint3
     return;
   }
   const uint32_t old = atomicMin(&s.t_vals[slot], j);
-  if (old < j) to_reduce(s, j, reduce_count, heavy_count, heavy_list);
-  else if (old != 0xFFFFFFFFu && old != j) to_reduce(s, old, reduce_count, heavy_count, heavy_list);
+  if (old < j) to_reduce(s, j, reduce_count, heavy);
+  else if (old != 0xFFFFFFFFu && old != j) to_reduce(s, old, reduce_count, heavy);
 }
 
 // owner of column j's current pivot in the table, which must precede j
@@ -837,7 +856,7 @@ __device__ __forceinline__ int64_t reduce_owner(const DimArgs& a, const RedState
 // the claim list unless it became zero.
 template <int D>
 __device__ void reduce_one(const DimArgs& a, const RedState& s, const Binom& B, int lane, const SortTile& tile,
-                           uint32_t j, uint32_t* claim_count, uint32_t* heavy_count, uint32_t* heavy_list) {
+                           uint32_t j, uint32_t* claim_count, const HeavyList& heavy) {
   uint64_t jidx;
   uint32_t jr, cl;
   column_simplex(a, s, j, &jidx, &jr, &cl);
@@ -850,7 +869,7 @@ __device__ void reduce_one(const DimArgs& a, const RedState& s, const Binom& B, 
   }
   const int st = chain_warp<D>(a, s, cv, B, lane, tile, j, jidx, jr, cl, a.chain_limit, ch);
   if (st == CH_HEAVY) {
-    chain_give_up(s, lane, j, heavy_count, heavy_list);
+    chain_give_up(s, lane, j, heavy);
     return;
   }
   if (st != CH_DONE) {
@@ -953,7 +972,8 @@ constexpr unsigned SUSP_LARGE = 0x80000000u;
 // reduce, ctl[16..17] heavy); ctl[4..5] are the barrier's counter and
 // generation, ctl[6] receives the number of rounds, ctl[12] is the progress
 // heartbeat, ctl[18..19] the light and heavy work cursors; ctl[20..22] count
-// the suspended columns (listed from ctl[64] on) and ctl[24..26] the teams done.
+// the suspended columns (listed from ctl[64] on) and ctl[24..26] the teams done;
+// ctl[28..29] tell, by round parity, of columns stored with many rows (HeavyList).
 template <int D>
 __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, RedState s, unsigned* ctl) {
   extern __shared__ uint64_t smem[];
@@ -984,8 +1004,10 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
   unsigned* heavy_next = ctl + 19;
   unsigned* susp_cnt = ctl + 20;
   unsigned* team_done = ctl + 24;
+  unsigned* large = ctl + 28;
   unsigned* susp_list = ctl + 64;
   uint32_t* heavy[2] = {s.heavy_list, s.heavy_list + (size_t)s.ncols + 1};
+  const auto heavies = [&](int q) { return HeavyList{heavy_cnt + q, heavy[q], large + q}; };
   const uint32_t ncols = s.ncols_dev ? *s.ncols_dev : s.ncols;
 
   // Additions a warp makes on a column in this phase: a few while its coboundaries fit the warp's tile, else none
@@ -993,7 +1015,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
   const bool tiles = s.scr_slice <= SORT_TILE;
   const uint32_t first_limit = tiles ? min(a.chain_limit, FIRST_CHAIN) : 0u;
   for (uint32_t j = warp_id; j < ncols; j += warps)
-    init_column<D>(a, s, B, lane, tile, j, first_limit, &claim_cnt[0], &heavy_cnt[0], heavy[0]);
+    init_column<D>(a, s, B, lane, tile, j, first_limit, &claim_cnt[0], heavies(0));
   if (!grid_barrier(bar_count, bar_gen, s, a.err)) return;
   uint32_t r = 0, it = 0;
   for (;; ++r) {
@@ -1009,9 +1031,10 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
     if ((nclaim == 0 && nqueued == 0) || (errs & (ERRF_ARENA | ERRF_TIMEOUT | ERRF_INTERNAL | ERRF_TABLE_FULL)))
       break;
     for (uint32_t t = tid; t < nclaim; t += threads)
-      claim_one(a, s, s.claim_list[t], &red_cnt[src], &heavy_cnt[src], heavy[src]);
+      claim_one(a, s, s.claim_list[t], &red_cnt[src], heavies(src));
     if (tid == 0) {  // the next round's heavy list and this round's cursors start empty
       heavy_cnt[dst] = 0;
+      large[dst] = 0;
       *light_next = 0;
       *heavy_next = 0;
     }
@@ -1027,12 +1050,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
     const uint32_t nlight = few ? 0u : nred;
     // no more than one column for two blocks, and one of them stored with so many rows that it takes a block long to
     // enter them: a team each from the start
-    bool direct = nlight == 0 && 2 * nwide <= gridDim.x;
-    if (direct) {
-      const uint32_t j = threadIdx.x < nheavy ? heavy[src][threadIdx.x]
-                         : threadIdx.x < nwide ? s.reduce_list[threadIdx.x - nheavy] : 0u;
-      direct = __syncthreads_or(threadIdx.x < nwide && s.r_len[j] > TEAM_MIN_ROWS);
-    }
+    bool direct = nlight == 0 && 2 * nwide <= gridDim.x && *(volatile unsigned*)&large[src];
     if (direct && blockIdx.x < nwide && threadIdx.x == 0) {
       WideCtx* c = s.wide + blockIdx.x;
       const int ph = ws.ph;
@@ -1061,7 +1079,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
           if (lane == 0) t = nlight ? atomicAdd(light_next, 1u) : 0u;
           t = __shfl_sync(0xffffffffu, t, 0);
           if (t >= nlight) break;
-          reduce_one<D>(a, s, B, lane, tile, s.reduce_list[t], &claim_cnt[dst], &heavy_cnt[dst], heavy[dst]);
+          reduce_one<D>(a, s, B, lane, tile, s.reduce_list[t], &claim_cnt[dst], heavies(dst));
         }
         if (!grid_barrier(bar_count, bar_gen, s, a.err)) return;
       }

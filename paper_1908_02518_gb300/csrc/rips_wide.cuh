@@ -64,7 +64,6 @@ constexpr uint32_t WIDE_K0 = 8;         // rows of the first window
 // over Z/3 15.7 -> 16.6).
 constexpr uint32_t WIDE_TEAM_K0 = 32, WIDE_TEAM_K1 = 512;
 constexpr uint32_t WIDE_SAMPLES = 128;   // keys sampled to place a bound, one a thread
-constexpr uint32_t TEAM_MIN_ROWS = 1024;  // stored rows from which a column starts with a team
 constexpr uint32_t TEAM_MIN_STEPS = 32;  // additions a block makes before it gives its column to a team
 constexpr uint32_t TEAM_SMALL = 64;         // blocks of a lone team up to
 constexpr uint32_t TEAM_LARGE_STEPS = 4096;  // additions

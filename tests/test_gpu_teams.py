@@ -34,3 +34,20 @@ def test_columns_that_change_teams(oracle_mod, name, make, dim_max, t, p, chain)
         res = rg.barcodes(x, dim_max, t, p)
         assert max(s["longest_chain"] for s in res.stats[0]) >= chain
         assert _key(res.bars) == want
+
+
+def test_columns_that_start_with_a_team(oracle_mod):
+    """A few columns left, with thousands of stored rows (a circle's last ones):
+    a team each from the start of the round, which all blocks have to agree on."""
+    import torch
+    import numpy as np
+    import paper_1908_02518_gb300 as rg
+    clouds = [W.circle_points(np.random.Generator(np.random.PCG64(s)), n).astype(np.float32)
+              for s, n in ((5, 150), (6, 149), (7, 33), (8, 128))]
+    off = np.cumsum([0] + [len(c) for c in clouds])
+    x = torch.from_numpy(np.concatenate(clouds)).cuda()
+    want = [_key(oracle_mod.barcodes(W.distance_matrix(c), 1).bars) for c in clouds]
+    for _ in range(10):
+        res = rg.barcodes_batched(x, off, 1)
+        for c in range(len(clouds)):
+            assert _key(res.bars[res.bars["cloud"] == c]) == want[c], c
