@@ -1028,8 +1028,8 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
     if (threadIdx.x == 0) errs_seen = *(volatile uint32_t*)a.err;
     __syncthreads();
     const uint32_t errs = errs_seen;
-    if ((nclaim == 0 && nqueued == 0) || (errs & (ERRF_ARENA | ERRF_TIMEOUT | ERRF_INTERNAL | ERRF_TABLE_FULL)))
-      break;
+    // (a full table is only found by claims, which other blocks may be at: seen after them)
+    if ((nclaim == 0 && nqueued == 0) || (errs & (ERRF_ARENA | ERRF_TIMEOUT | ERRF_INTERNAL))) break;
     for (uint32_t t = tid; t < nclaim; t += threads)
       claim_one(a, s, s.claim_list[t], &red_cnt[src], heavies(src));
     if (tid == 0) {  // the next round's heavy list and this round's cursors start empty
@@ -1039,6 +1039,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
       *heavy_next = 0;
     }
     if (!grid_barrier(bar_count, bar_gen, s, a.err)) return;
+    if (*(volatile uint32_t*)a.err & ERRF_TABLE_FULL) break;
     if (tid == 0) {
       claim_cnt[src] = 0;
       red_cnt[dst] = 0;

@@ -51,3 +51,27 @@ def test_columns_that_start_with_a_team(oracle_mod):
         res = rg.barcodes_batched(x, off, 1)
         for c in range(len(clouds)):
             assert _key(res.bars[res.bars["cloud"] == c]) == want[c], c
+
+
+def test_a_full_table_ends_all_blocks_together():
+    """A claim that finds the pivot table full is seen by every block at the same
+    point: none is left at a barrier until its wait runs out (30 s, and a timeout
+    status)."""
+    import time
+    import torch
+    import paper_1908_02518_gb300 as rg
+    from paper_1908_02518_gb300 import _lib
+    x = torch.from_numpy(W.distance_matrix(W.sphere_points(64, 1005, 4))).cuda()
+    want = _key(rg.barcodes(x, 3, math.inf, 3).bars)
+    try:
+        for slots in (16, 32, 64):
+            rg.set_limits(table_slots=slots)
+            for _ in range(10):
+                t0 = time.monotonic()
+                with pytest.raises(_lib.RipsError) as e:
+                    rg.barcodes(x, 3, math.inf, 3)
+                assert e.value.status == -4  # RIPS_ERR_OOM
+                assert time.monotonic() - t0 < 10
+    finally:
+        rg.set_limits()
+    assert _key(rg.barcodes(x, 3, math.inf, 3).bars) == want
