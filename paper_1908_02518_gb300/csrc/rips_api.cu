@@ -823,13 +823,13 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       CK(cudaMemcpyAsync(&hp->u32[16], counts, 64, cudaMemcpyDeviceToHost, s));
       CK(cudaMemcpyAsync(&hp->u32[8], w.err.p, 4, cudaMemcpyDeviceToHost, s));
       CR(sync_read(w, s));
+      if (int e = map_device_error(hp->u32[8])) return e;  // whatever else failed, with a full arena or not
       if (hp->u32[8] & ERRF_ARENA) {
         // start this dimension's reduction over with a larger arena (the readout of a failed one writes nothing)
         CK(cudaMemsetAsync(w.err.p, 0, 4, s));
         rcap *= 8;
         continue;
       }
-      if (int e = map_device_error(hp->u32[8])) return e;
       out.stats.resize((size_t)C * (dim_max + 1));
       // rounds and steps are properties of the whole batch's reduction
       const uint32_t* hc = &hp->u32[16];
@@ -1500,8 +1500,8 @@ int plan_result(PlanState& pl, cudaStream_t s, rips_result_t** out) {
   uint32_t err = 0;
   CK(cudaStreamSynchronize(s));
   CK(cudaMemcpy(&err, w.err.p, 4, cudaMemcpyDeviceToHost));
-  if (err & ERRF_ARENA) return RIPS_ERR_OOM;  // the plan's arena is fixed: make the plan with a larger one
   if (int e = map_device_error(err)) return e;
+  if (err & ERRF_ARENA) return RIPS_ERR_OOM;  // the plan's arena is fixed: make the plan with a larger one
   // one more wait: counters and statistics, and as many of the bars, in order, as the small sort takes
   const uint32_t most = (uint32_t)std::min<size_t>(bar_order_small_most(), w.bars.cap / sizeof(rips_bar_t));
   const size_t bars_at = 256, st_at = bars_at + (size_t)most * sizeof(rips_bar_t),

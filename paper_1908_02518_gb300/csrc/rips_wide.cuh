@@ -144,15 +144,17 @@ __device__ bool wide_sync(const Team& t, const RedState& s, WideState& w) {
 }
 
 // count arena entries for the team, from a multiple of four on (16-byte loads of
-// keys and coefficients); false when the arena is full
-__device__ bool wide_alloc(const Team& t, const RedState& s, WideState& w, unsigned long long count, WideList* out) {
+// keys and coefficients): CH_DONE, CH_ARENA when the arena is full, CH_LONG when the
+// wait for the team ran out (so for all that allocates below)
+__device__ int wide_alloc(const Team& t, const RedState& s, WideState& w, unsigned long long count, WideList* out) {
   if (threadIdx.x == 0 && t.rank == 0) {
     const unsigned long long o = (atomicAdd(s.r_top, count + 3) + 3) & ~3ull;
     *(volatile unsigned long long*)&t.g->c[w.ph].tmp = o + count <= s.r_cap ? o : ~0ull;
   }
-  if (!wide_sync(t, s, w) || w.d.tmp == ~0ull) return false;
+  if (!wide_sync(t, s, w)) return CH_LONG;
+  if (w.d.tmp == ~0ull) return CH_ARENA;
   *out = WideList{w.d.tmp, count};
-  return true;
+  return CH_DONE;
 }
 
 // ---------------------------------------------------------------- lists and table
@@ -320,21 +322,21 @@ __device__ __forceinline__ unsigned wide_insert(const RedState& s, const WideSta
 }
 
 // the list's other buffer holds at least `cap` entries
-__device__ bool wide_alt(const Team& t, const RedState& s, WideState& w, int l, unsigned long long cap) {
-  if (w.list[l][w.cur[l] ^ 1].cap >= cap) return true;
+__device__ int wide_alt(const Team& t, const RedState& s, WideState& w, int l, unsigned long long cap) {
+  if (w.list[l][w.cur[l] ^ 1].cap >= cap) return CH_DONE;
   WideList nl;
-  if (!wide_alloc(t, s, w, cap + cap / 2 + 64, &nl)) return false;
+  if (const int e = wide_alloc(t, s, w, cap + cap / 2 + 64, &nl)) return e;
   if (threadIdx.x == 0) w.list[l][w.cur[l] ^ 1] = nl;
   __syncthreads();
-  return true;
+  return CH_DONE;
 }
 
 // room for `room` more rows in list l
-__device__ bool wide_room(const Team& t, const RedState& s, WideState& w, int l, unsigned long long room) {
+__device__ int wide_room(const Team& t, const RedState& s, WideState& w, int l, unsigned long long room) {
   const uint32_t n = w.n[l];
   const WideList old = w.list[l][w.cur[l]];
-  if (n + room <= old.cap) return true;
-  if (!wide_alt(t, s, w, l, n + room)) return false;
+  if (n + room <= old.cap) return CH_DONE;
+  if (const int e = wide_alt(t, s, w, l, n + room)) return e;
   const WideList to = w.list[l][w.cur[l] ^ 1];
   if (n) {
     const uint32_t step = (uint32_t)t.size * blockDim.x;
@@ -342,20 +344,20 @@ __device__ bool wide_room(const Team& t, const RedState& s, WideState& w, int l,
       s.r_key[to.off + i] = __ldcg(s.r_key + old.off + i);
       if (l == L_FRONT) s.r_coef[to.off + i] = __ldcg(s.r_coef + old.off + i);
     }
-    if (!wide_sync(t, s, w)) return false;
+    if (!wide_sync(t, s, w)) return CH_LONG;
   } else {
     __syncthreads();  // every thread has read cur
   }
   if (threadIdx.x == 0) w.cur[l] ^= 1;
   __syncthreads();
-  return true;
+  return CH_DONE;
 }
 
 // an empty table of `cap` (a power of two >= 1024) slots in the other table buffer
-__device__ bool wide_table(const Team& t, const RedState& s, WideState& w, unsigned long long cap) {
+__device__ int wide_table(const Team& t, const RedState& s, WideState& w, unsigned long long cap) {
   if (w.tab[w.tcur ^ 1].cap < cap) {
     WideList nl;
-    if (!wide_alloc(t, s, w, cap, &nl)) return false;
+    if (const int e = wide_alloc(t, s, w, cap, &nl)) return e;
     if (threadIdx.x == 0) w.tab[w.tcur ^ 1] = nl;
     __syncthreads();
   }
@@ -366,7 +368,7 @@ __device__ bool wide_table(const Team& t, const RedState& s, WideState& w, unsig
   const unsigned long long first = (unsigned long long)t.rank * blockDim.x + threadIdx.x;
   for (unsigned long long i = first; i < cap / 2; i += step) tk[i] = make_ulonglong2(IDX_NONE, IDX_NONE);
   for (unsigned long long i = first; i < cap / 4; i += step) tv[i] = make_uint4(0, 0, 0, 0);
-  return wide_sync(t, s, w);
+  return wide_sync(t, s, w) ? CH_DONE : CH_LONG;
 }
 
 __device__ __forceinline__ unsigned long long wide_pow2(unsigned long long x) {
@@ -415,7 +417,7 @@ __device__ __forceinline__ bool wide_live(uint32_t v, uint32_t p) { return p == 
 __device__ int wide_ensure(const Team& t, const RedState& s, WideState& w, uint32_t p, unsigned long long room) {
   const int lane = threadIdx.x & 31;
   for (int l = 0; l < 2; ++l)
-    if (!wide_room(t, s, w, l, room)) return CH_ARENA;
+    if (const int e = wide_room(t, s, w, l, room)) return e;
   // (the second time unless a quarter of that is left free, or the next section would be back here)
   bool rebuilt = false;
   while (2 * (w.used + room) > (rebuilt ? (w.tmask + 1) / 4 * 3 : w.tmask + 1)) {
@@ -433,8 +435,8 @@ __device__ int wide_ensure(const Team& t, const RedState& s, WideState& w, uint3
     }
     const unsigned long long cap = wide_pow2(need);
     if (cap > (1ull << 32)) return CH_ARENA;
-    if (!wide_table(t, s, w, cap)) return CH_ARENA;
-    if (!wide_alt(t, s, w, L_MID, w.n[L_MID] + room)) return CH_ARENA;
+    if (const int e = wide_table(t, s, w, cap)) return e;
+    if (const int e = wide_alt(t, s, w, L_MID, w.n[L_MID] + room)) return e;
     const unsigned long long from = w.tab[w.tcur].off, to = w.tab[w.tcur ^ 1].off;
     const uint64_t fmask = w.tmask, tmask = cap - 1, bound = w.bound;
     const unsigned long long foff = w.list[L_FRONT][w.cur[L_FRONT]].off, moff = w.list[L_MID][w.cur[L_MID]].off;
@@ -568,9 +570,10 @@ __device__ int wide_split(const Team& t, const RedState& s, WideState& w, int l,
                           uint64_t settled = 0) {
   const int lane = threadIdx.x & 31;
   const uint32_t n = w.n[l];
-  if (!wide_alt(t, s, w, l, n)) return CH_ARENA;
+  if (const int e = wide_alt(t, s, w, l, n)) return e;
   for (int q = 0; q < 2; ++q)
-    if (q != l && (q == lo || q == hi) && !wide_room(t, s, w, q, n)) return CH_ARENA;
+    if (q != l && (q == lo || q == hi))
+      if (const int e = wide_room(t, s, w, q, n)) return e;
   const unsigned long long off = w.list[l][w.cur[l]].off;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -624,7 +627,7 @@ __device__ int wide_refill(const Team& t, const RedState& s, WideState& w, uint3
     const uint64_t after = w.mbound;
     if (after == ~0ull) return CH_MERGE;
     const uint64_t b = wide_sample_table(s, w, p, after, 8 * k, sm);
-    if (!wide_room(t, s, w, L_MID, w.used)) return CH_ARENA;
+    if (const int e = wide_room(t, s, w, L_MID, w.used)) return e;
     __syncthreads();
     if (threadIdx.x == 0) w.mbound = b;
     __syncthreads();
@@ -980,7 +983,7 @@ __device__ __forceinline__ int wide_begin(const DimArgs& a, const RedState& s, c
   if (w.lng.cap == 0) {  // a first column: its buffers in one piece
     const unsigned long long cap0 = wide_pow2(2 * (own + (unsigned long long)WIDE_K0 * s.scr_slice)), row = cap0 / 2;
     WideList nl;
-    if (!wide_alloc(t, s, w, cap0 + 4 * row + 4 * WIDE_LONGS, &nl)) return CH_ARENA;
+    if (const int e = wide_alloc(t, s, w, cap0 + 4 * row + 4 * WIDE_LONGS, &nl)) return e;
     if (threadIdx.x == 0) {
       unsigned long long o = nl.off;
       w.tab[w.tcur ^ 1] = WideList{o, cap0};
@@ -993,7 +996,8 @@ __device__ __forceinline__ int wide_begin(const DimArgs& a, const RedState& s, c
     __syncthreads();
   }
   const unsigned long long cap = wide_pow2(2 * (own + (unsigned long long)WIDE_K0 * s.scr_slice));
-  if (cap > (1ull << 32) || !wide_table(t, s, w, cap)) return CH_ARENA;
+  if (cap > (1ull << 32)) return CH_ARENA;
+  if (const int e = wide_table(t, s, w, cap)) return e;
   __syncthreads();
   if (threadIdx.x == 0) {
     w.tcur ^= 1;
@@ -1058,10 +1062,13 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
       }
     }
     const uint32_t nm = extend ? w.n[L_MID] : 0u;
-    if (extend && (!wide_alt(t, s, w, L_MID, nm) || !wide_room(t, s, w, L_FRONT, nm))) return CH_ARENA;
+    if (extend) {
+      if (const int e = wide_alt(t, s, w, L_MID, nm)) return e;
+      if (const int e = wide_room(t, s, w, L_FRONT, nm)) return e;
+    }
     if (w.todo.cap < 2ull * (w.n[L_FRONT] + nm)) {
       WideList nl;
-      if (!wide_alloc(t, s, w, 3ull * (w.n[L_FRONT] + nm) + 64, &nl)) return CH_ARENA;
+      if (const int e = wide_alloc(t, s, w, 3ull * (w.n[L_FRONT] + nm) + 64, &nl)) return e;
       if (threadIdx.x == 0) w.todo = nl;
       __syncthreads();
     }
@@ -1164,7 +1171,7 @@ __device__ __forceinline__ int wide_finish(const DimArgs& a, const RedState& s, 
   uint32_t len = 0;
   if (w.step && piv != IDX_NONE) {
     const uint32_t step = (uint32_t)t.size * blockDim.x, first = (uint32_t)t.rank * blockDim.x + threadIdx.x;
-    if (!wide_alt(t, s, w, L_MID, w.used)) return CH_ARENA;
+    if (const int e = wide_alt(t, s, w, L_MID, w.used)) return e;
     const WideView v = wide_view(t, w);
     const unsigned long long buf = w.list[L_MID][w.cur[L_MID] ^ 1].off;
     wide_scan(t, s, v.toff, v.mask + 1, [&](const uint64_t (&key)[8], const uint32_t (&val)[8]) {
@@ -1189,7 +1196,7 @@ __device__ __forceinline__ int wide_finish(const DimArgs& a, const RedState& s, 
     if (!wide_sync(t, s, w)) return CH_LONG;
     len = w.d.count;
     WideList run;
-    if (!wide_alloc(t, s, w, len, &run)) return CH_ARENA;
+    if (const int e = wide_alloc(t, s, w, len, &run)) return e;
     roff = run.off;
     if (sorted && len <= SORT_RUN) {
       if (t.rank == 0) {

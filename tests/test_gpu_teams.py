@@ -75,3 +75,26 @@ def test_a_full_table_ends_all_blocks_together():
     finally:
         rg.set_limits()
     assert _key(rg.barcodes(x, 3, math.inf, 3).bars) == want
+
+
+def test_a_wait_that_runs_out_is_a_timeout_with_a_full_arena_too():
+    """A reduction whose waits run out is not started over in a larger arena, also
+    when the arena was full at that time: as many launches as with room."""
+    import torch
+    import paper_1908_02518_gb300 as rg
+    from paper_1908_02518_gb300 import _lib
+    x = torch.from_numpy(W.distance_matrix(W.torus_points(300, 21))).cuda()
+    want = _key(rg.barcodes(x, 2, 1.2).bars)
+    launches = []
+    try:
+        for entries in (0, 64):
+            rg.set_limits(barrier_wait_ns=1, chain_ns=1, arena_entries=entries)
+            rg.launch_count(reset=True)
+            with pytest.raises(_lib.RipsError) as e:
+                rg.barcodes(x, 2, 1.2)
+            assert e.value.status == -6  # RIPS_ERR_DEVICE_TIMEOUT
+            launches.append(rg.launch_count())
+    finally:
+        rg.set_limits()
+    assert launches[1] <= launches[0]
+    assert _key(rg.barcodes(x, 2, 1.2).bars) == want
