@@ -399,7 +399,9 @@ RIPS_API uint32_t rips_get_options(void);
  * The reduction's arena is fixed too: arena_entries entries of 12 bytes (0:
  * 384 per edge, within 40 % of the free device memory) for stored columns, and
  * beside them, as far as the 40 % leave room, the tables and lists of the columns
- * under way (at most 1664 per edge); a run that needs more
+ * under way: at most 640 per edge or twice arena_entries, whichever is more.  So
+ * arena_entries bounds a plan's memory, down to 640 entries per edge; a run that
+ * needs more than it has
  * reports RIPS_ERR_OOM from rips_batch_plan_result.  A plan is used by one
  * stream at a time. */
 typedef struct rips_batch_plan rips_batch_plan_t;

@@ -35,13 +35,14 @@ struct Buf {
   size_t cap = 0;
 };
 
-static int ensure(Buf& b, size_t bytes) {
+// `roomy`: with a quarter more, for buffers that grow from call to call
+static int ensure(Buf& b, size_t bytes, bool roomy = true) {
   if (bytes == 0) bytes = 8;
   if (bytes <= b.cap) return RIPS_OK;
   if (b.p) cudaFree(b.p);
   b.p = nullptr;
   b.cap = 0;
-  size_t want = bytes + bytes / 4;
+  size_t want = roomy ? bytes + bytes / 4 : bytes;
   if (cudaMalloc(&b.p, want) != cudaSuccess) {
     cudaGetLastError();
     if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
@@ -1314,9 +1315,13 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
     // the caller's entries, or 384 per edge within 40 % of free memory, for stored columns and generated coboundaries
     pl.arena = arena_entries ? (size_t)arena_entries
                              : std::max<size_t>(std::min<size_t>(384 * (size_t)pl.e_cap, fit), (size_t)1 << 22);
-    // and, as far as that leaves room within the 40 %, the tables and lists of the columns under way: a block's are a
-    // few tens of its first ones' size (96 entries a slot of a coboundary) by the time its columns have grown
-    const size_t tables = std::min<size_t>(1664 * (size_t)pl.e_cap, (size_t)3072 * pl.slice * (size_t)pl.blocks);
+    // and, as far as that leaves room within the 40 %, the tables and lists of the columns under way: 640 per edge
+    // where they are few to a block, or twice the caller's entries.  Both together were used up to 113 of them an edge
+    // by 256 clouds, 117 by 24 clouds of 64 to 128 points, 350 by 4 of 200 to 400, 620 by 3 of 600 to 800, 720 by a
+    // torus of 1,000; 500 rotations, whose columns grow to half of all rows, take 2,100.
+    const size_t tables = std::max<size_t>(arena_entries ? 2 * (size_t)arena_entries : 0,
+                                           std::min<size_t>(640 * (size_t)pl.e_cap,
+                                                            (size_t)3072 * pl.slice * (size_t)pl.blocks));
     if (pl.arena < fit) pl.arena += std::min(tables, fit - pl.arena);
   }
   Workspace& w = pl.w;
@@ -1363,8 +1368,8 @@ int plan_create(PlanState& pl, const int64_t* offsets, int32_t batch, int32_t k,
   CR(ensure(w.heavy, (E + 1) * 8));
   CR(ensure(w.lists, LISTS_BYTES));
   CR(ensure(w.r_top, 16));
-  CR(ensure(w.r_key, pl.arena * 8));
-  CR(ensure(w.r_coef, pl.arena * 4));
+  CR(ensure(w.r_key, pl.arena * 8, false));
+  CR(ensure(w.r_coef, pl.arena * 4, false));
   w.r_cap = pl.arena;
   if (cudaMemcpy(pl.clouds0.p, ci.data(), (size_t)batch * sizeof(CloudInfo), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(w.tileoff.p, vtile.data(), (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice) != cudaSuccess) {

@@ -987,9 +987,11 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
   __shared__ WideState ws, wt;  // this block's own column; the column of its team
   __shared__ WideShared wsh;
   __shared__ uint32_t take;
+  __shared__ bool lent;  // ws went into this block's context with a column, and is there again after the round
   uint64_t* const sm = (uint64_t*)red_smem;
   if (threadIdx.x == 0) {  // visible to the block after the first grid barrier
     ws = WideState{};
+    lent = false;
     for (int q = 0; q < 3; ++q) wide_clear(&wsh.c[q]);
   }
   const uint32_t w = threadIdx.x >> 5;
@@ -1049,6 +1051,16 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
     const bool few = !tiles || nred + nheavy <= BLOCK_COLUMNS * gridDim.x;  // blocks take all columns, a few each
     const uint32_t nwide = few ? nred + nheavy : nheavy;
     const uint32_t nlight = few ? 0u : nred;
+    if (lent) {  // the buffers of the column that this block gave to a team, with what it added
+      const int ph = ws.ph;
+      __syncthreads();
+      wide_load(&ws, &s.wide[blockIdx.x].st);
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        ws.ph = ph;
+        lent = false;
+      }
+    }
     // no more than one column for two blocks, and one of them stored with so many rows that it takes a block long to
     // enter them: a team each from the start
     bool direct = nlight == 0 && 2 * nwide <= gridDim.x && *(volatile unsigned*)&large[src];
@@ -1063,6 +1075,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
       susp_list[(it % 3) * gridDim.x + atomicAdd(&susp_cnt[it % 3], 1u)] = blockIdx.x;
       ws = WideState{};
       ws.ph = ph;
+      lent = true;
     }
     // Columns by blocks (queue), then light ones by warps, then what is suspended by teams.  A heavy column given up by
     // a warp may come with a pivot nobody owns yet; it then ends at once and claims it.
@@ -1109,7 +1122,7 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
         team.size = 0;  // none for this block
         if (q < nteam) {
           c = s.wide + (*(volatile unsigned*)&susp_list[(it % 3) * gridDim.x + q] & ~SUSP_LARGE);
-          if (threadIdx.x == 0) wt = c->st;
+          wide_load(&wt, &c->st);
           team = Team{(int)size, (int)(blockIdx.x - q * size), &c->sh};
         }
         const volatile unsigned* done = team_done + it % 3;
@@ -1136,19 +1149,15 @@ __global__ void __launch_bounds__(256, 2) reduce_persistent_kernel(DimArgs a, Re
             if (queue) {
               for (int q = 0; q < 3; ++q) wide_clear(&c->sh.c[q]);
               c->sh.bar_count = c->sh.bar_gen = 0;
-              const int ph = ws.ph;  // its buffers went with the column
+              const int ph = ws.ph;
               ws = WideState{};
               ws.ph = ph;
+              lent = true;
             }
           } else {
             if (!queue) atomicAdd(&team_done[it % 3], 1u);
-            if (st != CH_DONE) {
-              chain_error(a, st);
-            } else if (!queue && ws.tab[0].cap + ws.tab[1].cap == 0) {  // the buffers serve this block's next column
-              const int ph = ws.ph;
-              ws = wt;
-              ws.ph = ph;
-            }
+            if (st != CH_DONE) chain_error(a, st);
+            else if (!queue) c->st = w;  // the buffers go back to the block that began the column
           }
         }
         __syncthreads();

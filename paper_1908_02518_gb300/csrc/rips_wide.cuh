@@ -81,6 +81,13 @@ __device__ __forceinline__ void wide_clear(WideCount* c) {
   c->longsum = c->longroom = c->tmp = 0;
 }
 
+// a column's state from its context into shared memory, a word a thread
+__device__ __forceinline__ void wide_load(WideState* to, const WideState* from) {
+  static_assert(sizeof(WideState) % 4 == 0, "words");
+  for (uint32_t i = threadIdx.x; i < sizeof(WideState) / 4; i += blockDim.x)
+    ((unsigned*)to)[i] = ((const unsigned*)from)[i];
+}
+
 // Barrier of the team's blocks; bounded like the grid barrier.
 __device__ bool team_sync(const Team& t, const RedState& s) {
   if (t.size == 1) {
@@ -154,6 +161,31 @@ __device__ int wide_alloc(const Team& t, const RedState& s, WideState& w, unsign
   if (!wide_sync(t, s, w)) return CH_LONG;
   if (w.d.tmp == ~0ull) return CH_ARENA;
   *out = WideList{w.d.tmp, count};
+  return CH_DONE;
+}
+
+// `slot` (a buffer of w that holds nothing) becomes one of at least `need` entries:
+// the smallest of the spare ones that will do, or `count` new entries, and the old
+// one is kept as a spare.
+__device__ int wide_grow(const Team& t, const RedState& s, WideState& w, WideList& slot, unsigned long long need,
+                         unsigned long long count) {
+  int best = -1, least = 0;
+  for (int q = 0; q < WIDE_SPARES; ++q) {
+    const unsigned long long cap = w.spare[q].cap;
+    if (cap >= need && (best < 0 || cap < w.spare[best].cap)) best = q;
+    if (cap < w.spare[least].cap) least = q;
+  }
+  WideList nl = best >= 0 ? w.spare[best] : WideList{0, 0};
+  if (best < 0) {
+    if (const int e = wide_alloc(t, s, w, count, &nl)) return e;
+    if (slot.cap > w.spare[least].cap) best = least;  // the smallest one is given up
+  }
+  __syncthreads();  // every thread has read the spares
+  if (threadIdx.x == 0) {
+    if (best >= 0) w.spare[best] = slot;
+    slot = nl;
+  }
+  __syncthreads();
   return CH_DONE;
 }
 
@@ -323,12 +355,8 @@ __device__ __forceinline__ unsigned wide_insert(const RedState& s, const WideSta
 
 // the list's other buffer holds at least `cap` entries
 __device__ int wide_alt(const Team& t, const RedState& s, WideState& w, int l, unsigned long long cap) {
-  if (w.list[l][w.cur[l] ^ 1].cap >= cap) return CH_DONE;
-  WideList nl;
-  if (const int e = wide_alloc(t, s, w, cap + cap / 2 + 64, &nl)) return e;
-  if (threadIdx.x == 0) w.list[l][w.cur[l] ^ 1] = nl;
-  __syncthreads();
-  return CH_DONE;
+  WideList& alt = w.list[l][w.cur[l] ^ 1];
+  return alt.cap >= cap ? CH_DONE : wide_grow(t, s, w, alt, cap, cap + cap / 2 + 64);
 }
 
 // room for `room` more rows in list l
@@ -355,12 +383,8 @@ __device__ int wide_room(const Team& t, const RedState& s, WideState& w, int l, 
 
 // an empty table of `cap` (a power of two >= 1024) slots in the other table buffer
 __device__ int wide_table(const Team& t, const RedState& s, WideState& w, unsigned long long cap) {
-  if (w.tab[w.tcur ^ 1].cap < cap) {
-    WideList nl;
-    if (const int e = wide_alloc(t, s, w, cap, &nl)) return e;
-    if (threadIdx.x == 0) w.tab[w.tcur ^ 1] = nl;
-    __syncthreads();
-  }
+  if (w.tab[w.tcur ^ 1].cap < cap)
+    if (const int e = wide_grow(t, s, w, w.tab[w.tcur ^ 1], cap, cap)) return e;
   const unsigned long long off = w.tab[w.tcur ^ 1].off;
   const unsigned long long step = (unsigned long long)t.size * blockDim.x;
   ulonglong2* tk = (ulonglong2*)(s.r_key + off);
@@ -1067,10 +1091,8 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
       if (const int e = wide_room(t, s, w, L_FRONT, nm)) return e;
     }
     if (w.todo.cap < 2ull * (w.n[L_FRONT] + nm)) {
-      WideList nl;
-      if (const int e = wide_alloc(t, s, w, 3ull * (w.n[L_FRONT] + nm) + 64, &nl)) return e;
-      if (threadIdx.x == 0) w.todo = nl;
-      __syncthreads();
+      const unsigned long long rows = w.n[L_FRONT] + nm;
+      if (const int e = wide_grow(t, s, w, w.todo, 2 * rows, 3 * rows + 64)) return e;
     }
     const unsigned long long moff = w.list[L_MID][w.cur[L_MID]].off;
     __syncthreads();

@@ -10,6 +10,8 @@ struct WideList {
   unsigned long long off, cap;  // arena entries [off, off + cap)
 };
 
+constexpr int WIDE_SPARES = 4;
+
 // what a team's threads count during one section (between two team barriers)
 struct WideCount {
   unsigned add[2];  // rows appended to each list
@@ -40,6 +42,7 @@ struct WideState {
   WideList list[2][2];
   WideList tab[2];
   WideList todo, lng;
+  WideList spare[WIDE_SPARES];  // buffers outgrown by their list or table
   uint64_t tmask, used;
   uint64_t bound, mbound;
   unsigned long long t0;
