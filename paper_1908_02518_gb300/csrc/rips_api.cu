@@ -94,7 +94,7 @@ struct Workspace {
   std::mutex mu;
   int device = -1;
   Buf dist, binom, rowmax, teff, err, ecount;
-  Buf ekeys, ekeys_alt, eflags, escan, erank, rvalue, R, deg, nbr;
+  Buf ekeys, ekeys_alt, eflags, erank, rvalue, R, deg, nbr;
   Buf eu, ev, comp, best, parent, gtop, inforest, fpos, nf;
   Buf sidx[2], srank[2], scount;
   Buf ckeys, ckeys_alt, ccount, sorttmp;
@@ -1229,7 +1229,7 @@ void release(Buf& b) {
 void release_plan(PlanState& pl) {
   Workspace& w = pl.w;
   Buf* all[] = {&w.dist, &w.binom, &w.rowmax, &w.teff, &w.err, &w.ecount, &w.ekeys, &w.ekeys_alt, &w.eflags,
-                &w.escan, &w.erank, &w.rvalue, &w.R, &w.deg, &w.nbr, &w.eu, &w.ev, &w.comp, &w.best, &w.parent,
+                &w.erank, &w.rvalue, &w.R, &w.deg, &w.nbr, &w.eu, &w.ev, &w.comp, &w.best, &w.parent,
                 &w.gtop, &w.inforest, &w.fpos, &w.nf, &w.sidx[0], &w.sidx[1], &w.srank[0], &w.srank[1],
                 &w.scount, &w.ckeys, &w.ckeys_alt, &w.ccount, &w.sorttmp, &w.piv_key, &w.piv_coef, &w.r_off,
                 &w.r_len, &w.reduced, &w.claim, &w.reduce, &w.heavy, &w.lists, &w.r_key, &w.r_coef, &w.r_top, &w.wide,

@@ -77,12 +77,6 @@ __device__ __forceinline__ uint32_t high_part(uint64_t x, int bits) { return bit
 
 // ---------------------------------------------------------------- simplex helpers
 
-struct Simplex {
-  int v[MAX_DIM + 2];  // vertices, decreasing
-  uint64_t idx;
-  uint32_t rank;
-};
-
 // largest v in [lo, hi] with C(v, k) <= N, by bisection
 __device__ __forceinline__ int max_vertex_bisect(const Binom& B, int k, int lo, int hi, uint64_t N) {
   while (lo < hi) {

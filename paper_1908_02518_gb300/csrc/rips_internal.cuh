@@ -37,35 +37,6 @@ enum : uint32_t {
 void note_launch();
 
 // ------------------------------------------------------------------ device helpers
-__device__ __forceinline__ uint64_t binom(const uint64_t* __restrict__ tab, int stride, int i, int k) {
-  return tab[(size_t)k * stride + i];
-}
-
-// Largest v in [lo, hi] with C(v, k) <= N (the Lemma of Section 4,
-// "Vertices and simplices"), by binary search.  Requires C(lo, k) <= N.
-__device__ __forceinline__ int max_vertex(const uint64_t* __restrict__ tab, int stride, int lo, int hi,
-                                          int k, uint64_t N) {
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (binom(tab, stride, mid, k) <= N) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// Vertices of the d-simplex with index N, written in decreasing order
-// v[0] > v[1] > ... > v[d].
-__device__ __forceinline__ void decode_simplex(const uint64_t* __restrict__ tab, int stride, int n,
-                                               uint64_t N, int d, int* v) {
-  int hi = n - 1;
-  for (int k = d + 1; k >= 1; --k) {
-    int x = max_vertex(tab, stride, k - 1, hi, k, N);
-    v[d + 1 - k] = x;
-    N -= binom(tab, stride, x, k);
-    hi = x - 1;
-  }
-}
-
 // Z/p helpers (p < 2^16 so products fit in 32 bits)
 __device__ __forceinline__ uint32_t mod_inv(uint32_t a, uint32_t p) {
   // extended Euclid on (a, p), p prime, a != 0
@@ -286,7 +257,7 @@ cudaError_t launch_test(const DimArgs& a, const uint64_t* sidx, const uint32_t* 
 size_t wide_ctx_bytes(int blocks);
 // blocks of the cooperative reduction launch (all co-resident), -1 on error
 int reduction_blocks(const DimArgs& a, uint32_t ncols);
-// ctl: 8 zeroed uint32 (see reduce_persistent_kernel); ctl[6] receives the rounds
+// ctl: the control block, LISTS_BYTES of zeros (see reduce_persistent_kernel); ctl[6] receives the rounds
 cudaError_t launch_reduction(const DimArgs& a, const RedState& s, int blocks, unsigned* ctl, cudaStream_t st);
 // stats: [0] pairs, [1] zero pairs, [2] essential, [3] emergent per cloud
 cudaError_t launch_readout(const DimArgs& a, const RedState& s, const float* rank_value, rips_bar_t* bars,

@@ -103,20 +103,12 @@ struct Coboundary {
   }
 };
 
-// Apparent facet of the pivot row tau (a (d+1)-simplex): returns the facet's
-// reference (IDX_NONE if none; packed vertices when the pair map holds them,
-// see DimArgs::vbits, else its index), its rank and the coefficient of tau in
-// its coboundary.
-__device__ uint64_t pivot_apparent_facet(const DimArgs& a, const CV& cv, const Binom& B, int lane, uint32_t cl,
-                                         uint64_t key, uint32_t* frank, uint32_t* tcoef) {
+// Apparent facet of the pivot row tau (a (d+1)-simplex), for want of a pair map:
+// returns the facet's index (IDX_NONE if none), its rank and the coefficient of
+// tau in its coboundary.
+__device__ uint64_t pivot_apparent_facet(const DimArgs& a, const CV& cv, const Binom& B, int lane, uint64_t key,
+                                         uint32_t* frank, uint32_t* tcoef) {
   const int k = a.d + 1;
-  if (a.amap) {  // recorded by this dimension's test kernel
-    uint64_t v;
-    if (!pair_find(a.amap, a.amap_mask, table_key(a, cl, row_key_idx(a, key)), &v)) return IDX_NONE;
-    *frank = row_key_rank(a, key);
-    *tcoef = ((a.d - (int)(v & 15)) & 1) ? a.p - 1 : 1u;
-    return v >> 4;
-  }
   const uint64_t tidx = row_key_idx(a, key);
   const uint32_t tr = row_key_rank(a, key);
   int w[MAX_DIM + 2];
@@ -142,9 +134,9 @@ __device__ uint64_t pivot_apparent_facet(const DimArgs& a, const CV& cv, const B
 
 // Owner of the pivot row `key` of a column of cloud cl: the zero apparent facet
 // of the row (Section 4, "Persistence pairs": apparent pairs are not in the
-// table; its reference as pivot_apparent_facet gives it), else the table's
-// owner (0xFFFFFFFF: none).  With the recorded pair
-// map the two lookups run at once on lanes 0 and 1.  Warp-cooperative; every
+// table; its packed vertices when the pair map holds them, see DimArgs::vbits,
+// else its index), else the table's owner (0xFFFFFFFF: none).  With the recorded
+// pair map the two lookups run at once on lanes 0 and 1.  Warp-cooperative; every
 // lane gets the results.
 __device__ __forceinline__ uint64_t pivot_owner(const DimArgs& a, const RedState& s, const CV& cv, const Binom& B,
                                                 int lane, uint32_t cl, uint64_t key, uint32_t* frank, uint32_t* tcoef,
@@ -193,7 +185,7 @@ __device__ __forceinline__ uint64_t pivot_owner(const DimArgs& a, const RedState
     *tcoef = ((a.d - (int)(v & 15)) & 1) ? a.p - 1 : 1u;
     return v >> 4;
   }
-  const uint64_t fidx = pivot_apparent_facet(a, cv, B, lane, cl, key, frank, tcoef);
+  const uint64_t fidx = pivot_apparent_facet(a, cv, B, lane, key, frank, tcoef);
   *owner = 0xFFFFFFFFu;
   if (fidx == IDX_NONE) {
     const int64_t slot = table_find(s.t_keys, s.t_mask, tkey);
@@ -346,28 +338,15 @@ __device__ __forceinline__ Run empty_run() {
   return r;
 }
 
-// A run over n arena entries.  When the block has the first entries in shared
-// memory (sk, sc: the same keys and coefficients), the head and look-ahead are
-// taken from there instead of waiting for the arena.
+// a run over n arena entries
 __device__ __forceinline__ Run make_run(const uint64_t* k, const uint32_t* c, uint32_t n, uint32_t scale,
-                                        uint32_t p, const uint64_t* sk = nullptr, const uint32_t* sc = nullptr) {
+                                        uint32_t p) {
   Run r = empty_run();
   r.key = k;
   r.coef = c;
   r.len = n;
   r.scale = scale;
-  if (sk) {
-    r.hk = n ? sk[0] : ~0ull;
-    r.hc = n ? scaled(sc[0], scale, p) : 0u;
-#pragma unroll
-    for (int i = 0; i < RUN_AHEAD; ++i) {
-      const bool in = 1u + i < n;
-      r.nk[i] = in ? sk[1 + i] : ~0ull;
-      r.nc[i] = in ? sc[1 + i] : 1u;
-    }
-  } else {
-    run_head(r, p);
-  }
+  run_head(r, p);
   return r;
 }
 
@@ -560,24 +539,15 @@ struct Chain {
   unsigned long long t0;  // globaltimer when the chain passed 255 additions
 };
 
-enum : int { CH_DONE = 0, CH_MERGE = 1, CH_ARENA = 2, CH_LONG = 3, CH_INTERNAL = 4, CH_GEN = 5, CH_GEN_SELF = 6,
-             CH_HEAVY = 7 };
-
-// work handed from warp 0 to its block: runs to merge, or a coboundary to generate
-struct ChainReq {
-  unsigned mask;  // CH_MERGE: lanes of the runs
-  uint64_t gidx;  // CH_GEN, CH_GEN_SELF: the simplex (a reference as simplex_vertices takes it)
-  uint32_t grank;
-  bool gpacked;
-};
+// how a chain or one of its sections ends; CH_EMPTY: no rows left to look at
+enum : int { CH_DONE = 0, CH_EMPTY, CH_ARENA, CH_LONG, CH_HEAVY };
 
 // R_j <- R_j - lambda C, lambda = pivot coefficient ratio (Algorithm 1): the run
 // of C joins the set, then the new pivot is found
 __device__ __forceinline__ void chain_add(const DimArgs& a, const RedState& s, Chain& ch, int lane,
-                                          const uint64_t* wk, const uint32_t* wc, uint32_t wn, uint32_t wcoef,
-                                          const uint64_t* sk = nullptr, const uint32_t* sc = nullptr) {
+                                          const uint64_t* wk, const uint32_t* wc, uint32_t wn, uint32_t wcoef) {
   const uint32_t lam = (uint32_t)(((uint64_t)ch.coef * mod_inv(wcoef, a.p)) % a.p);
-  if (lane == ch.nr) ch.r = make_run(wk, wc, wn, (a.p - lam) % a.p, a.p, sk, sc);
+  if (lane == ch.nr) ch.r = make_run(wk, wc, wn, (a.p - lam) % a.p, a.p);
   ++ch.nr;
   ++ch.step;
   if (lane == 0) {

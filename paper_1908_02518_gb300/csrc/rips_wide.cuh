@@ -319,9 +319,11 @@ __device__ __forceinline__ WideView wide_view(const Team& t, const WideState& w)
 
 // Adds c (mod p) to row `key` of the working column, U rows a lane (where ok);
 // a row seen for the first time joins the list of its key.  Returns how many of
-// the lane's rows are new.  Sums of coefficients below p stay below 2^32: the
-// add that passes 2^31 takes a multiple of p off again (a row lies in at most
-// d + 2 coboundaries, so few adds of one row are ever under way at once).
+// the lane's rows are new.  Sums of coefficients below p < 2^16 stay below 2^32:
+// the add that passes 2^31 takes a multiple of p off again, and no more adds of one
+// row are under way at a time than there are warps in the team (an added column
+// has a row once, is added by one warp, and the warp waits for its adds): 2,432 of
+// less than 2^16 each on 304 blocks.
 template <int U>
 __device__ __forceinline__ unsigned wide_insert(const RedState& s, const WideState& w, const WideView& v, int lane,
                                                 uint32_t p, const bool (&ok)[U], const uint64_t (&key)[U],
@@ -642,14 +644,13 @@ __device__ int wide_split(const Team& t, const RedState& s, WideState& w, int l,
 
 // Rows in the mid list for the next part of the window, about k of them: the list
 // is refilled from the table with 8 k when it is empty, and cut down to them when
-// it has outgrown 24 k.  CH_MERGE (used as "no rows left") when nothing lies
-// beyond the front.
+// it has outgrown 24 k.  CH_EMPTY when nothing lies beyond the front.
 __device__ int wide_refill(const Team& t, const RedState& s, WideState& w, uint32_t p, unsigned long long k,
                            uint64_t* sm) {
   const int lane = threadIdx.x & 31;
   while (w.n[L_MID] == 0) {
     const uint64_t after = w.mbound;
-    if (after == ~0ull) return CH_MERGE;
+    if (after == ~0ull) return CH_EMPTY;
     const uint64_t b = wide_sample_table(s, w, p, after, 8 * k, sm);
     if (const int e = wide_room(t, s, w, L_MID, w.used)) return e;
     __syncthreads();
@@ -780,7 +781,7 @@ __device__ __forceinline__ uint64_t wide_look(const DimArgs& a, const RedState& 
       const int L = __ffs(m) - 1;
       m &= m - 1;
       uint32_t fr, tc;
-      const uint64_t fi = pivot_apparent_facet(a, cv, B, lane, w.cl, __shfl_sync(0xffffffffu, key, L), &fr, &tc);
+      const uint64_t fi = pivot_apparent_facet(a, cv, B, lane, __shfl_sync(0xffffffffu, key, L), &fr, &tc);
       if (lane == L) {
         if (fi == IDX_NONE) {
           code = wide_owner(a, s, w.cl, w.j, key);
@@ -1077,7 +1078,7 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
       if (e == CH_DONE) {
         extend = true;
         b = w.n[L_MID] <= 2 * want ? w.mbound : wide_sample(s, w, p, L_MID, want, sm);
-      } else if (e != CH_MERGE) {
+      } else if (e != CH_EMPTY) {
         return e;
       } else if (w.n[L_FRONT] == 0) {
         *piv = IDX_NONE;
