@@ -1150,6 +1150,8 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
         share = 0.0f;
         continue;
       }
+      // the bound stays: no block adds to the rows before all have sampled them, or it would find another bound
+      if (t.size > 1 && !wide_sync(t, s, w)) return CH_LONG;
     } else if (w.n[L_FRONT] > 4 * min((unsigned long long)k * w.dil, rows) + 1024) {  // mostly settled rows: drop them
       const int e = wide_split(t, s, w, L_FRONT, w.bound, L_FRONT, L_MID, ow);
       if (e != CH_DONE) return e;

@@ -98,3 +98,30 @@ def test_a_wait_that_runs_out_is_a_timeout_with_a_full_arena_too():
         rg.set_limits()
     assert launches[1] <= launches[0]
     assert _key(rg.barcodes(x, 2, 1.2).bars) == want
+
+
+def _uniform(n):
+    import numpy as np
+    a = np.tril(np.random.Generator(np.random.PCG64(n)).random((n, n)).astype(np.float32), -1)
+    return a + a.T
+
+
+def _hamming(n, bits):
+    import numpy as np
+    x = np.random.Generator(np.random.PCG64(n)).integers(0, 2, (n, bits))
+    return (x[:, None] != x[None]).sum(-1).astype(np.float32)
+
+
+@pytest.mark.parametrize("name,make,dim_max", [("uniform140", lambda: _uniform(140), 1),
+                                               ("uniform60", lambda: _uniform(60), 2),
+                                               ("hamming200", lambda: _hamming(200, 40), 1)])
+def test_lengths_without_geometry(oracle_mod, name, make, dim_max):
+    """Random lengths: rows come back as fast as they are eliminated, windows are cut
+    back time and again, and all blocks of a team have to cut them alike."""
+    import torch
+    import paper_1908_02518_gb300 as rg
+    d = make()
+    want = _key(oracle_mod.barcodes(d, dim_max).bars)
+    x = torch.from_numpy(d).cuda()
+    for _ in range(20):
+        assert _key(rg.barcodes(x, dim_max).bars) == want
