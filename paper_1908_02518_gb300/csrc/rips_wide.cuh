@@ -27,8 +27,10 @@
 // rounds and the additions wasted on rows past its pivot are a share of A: a
 // third of them and at least 8 for a block, since other columns wait for it; for
 // a team as many as made, between 32 and 512, and half as many beyond, since half
-// of the chip waits for a team and a round costs it a barrier over blocks more.  A
-// window whose rows multiply is cut back to K.  (K counts rows that have an
+// of the chip waits for a team and a round costs it a barrier over blocks more.
+// That holds while rows stay eliminated; K is therefore also bound by the rows
+// that rounds settle (WIDE_AHEAD).  A window whose rows multiply is cut back to K.
+// (K counts rows that have an
 // owner: the window is extended by the share of such rows the last time.)  Rows
 // behind the window are settled; a table that fills up is rebuilt from its live
 // rows.
@@ -63,6 +65,14 @@ constexpr uint32_t WIDE_K0 = 8;         // rows of the first window
 // clouds 24.9 -> 25.3 to 28.6, 100 points 0.75 -> 0.80 to 0.85), all additions past 512 too (3-sphere of 144 points
 // over Z/3 15.7 -> 16.6).
 constexpr uint32_t WIDE_TEAM_K0 = 32, WIDE_TEAM_K1 = 512;
+// And at most WIDE_AHEAD times the rows that a round has settled of late (rows older than every live one), or as many
+// as bring this many entries a block, whose additions a round's latency hides.  On lengths without geometry rows come
+// back as often as they are eliminated and a round settles about one, however wide the window: without this bound it
+// grows all the same.  Random lengths, 200 points 220 -> 105 ms (1.37 million additions -> 88,000), 300 points of 40
+// bits by Hamming distance 82 -> 38, integers up to 9 on 1,000 points 240 to 390 -> 58; with geometry 0.5 % slower.
+// 1,024 for teams: 89 and 31 ms, but 4,999 points of a Clifford torus 6 % slower; 16,384: 134 and 58.
+constexpr float WIDE_AHEAD = 4.0f;
+constexpr float WIDE_FREE = 1024.0f, WIDE_TEAM_FREE = 4096.0f;
 constexpr uint32_t WIDE_SAMPLES = 128;   // keys sampled to place a bound, one a thread
 constexpr uint32_t TEAM_MIN_STEPS = 32;  // additions a block makes before it gives its column to a team
 constexpr uint32_t TEAM_SMALL = 64;         // blocks of a lone team up to
@@ -76,7 +86,7 @@ struct Team {
 
 __device__ __forceinline__ void wide_clear(WideCount* c) {
   c->add[0] = c->add[1] = c->fresh = c->todo = 0;
-  c->count = c->nlong = c->stop = 0;
+  c->count = c->nlong = c->stop = c->settled = c->ents = 0;
   c->un = c->ow = ~0ull;
   c->longsum = c->longroom = c->tmp = 0;
 }
@@ -746,10 +756,15 @@ __device__ __forceinline__ uint64_t wide_owner(const DimArgs& a, const RedState&
   return OWN_NONE;
 }
 
-// new rows of a warp's lanes, counted once a section
-__device__ __forceinline__ void wide_count_fresh(WideCount* c, int lane, unsigned fresh) {
+// two neighbouring counts with one atomic
+__device__ __forceinline__ void wide_count2(unsigned* first, unsigned a, unsigned b) {
+  if (a | b) atomicAdd((unsigned long long*)first, a | ((unsigned long long)b << 32));
+}
+
+// new rows of a warp's lanes and the entries it added, counted once a section
+__device__ __forceinline__ void wide_count_fresh(WideCount* c, int lane, unsigned fresh, unsigned ents = 0) {
   fresh = __reduce_add_sync(0xffffffffu, fresh);
-  if (lane == 0 && fresh) atomicAdd(&c->fresh, fresh);
+  if (lane == 0) wide_count2(&c->fresh, fresh, ents);
 }
 
 // kinds of work records (two arena entries: key words ref, kind << 32 | length,
@@ -868,6 +883,8 @@ __device__ __forceinline__ void wide_check(const DimArgs& a, const RedState& s, 
   const uint32_t n = w.n[L_FRONT];
   const uint32_t p = a.p;
   WideSeen seen{~0ull, ~0ull, 0};
+  const uint64_t lo = w.lo, hi = w.hi;
+  unsigned settled = 0;
   const uint32_t ft = (n + 127) / 128, tiles = ft + (nm + 127) / 128;
   const uint32_t tw = (uint32_t)t.rank + (threadIdx.x >> 5) * (uint32_t)t.size, TW = (uint32_t)t.size * WARPS_PER_BLOCK;
   unsigned joined = 0;
@@ -890,6 +907,7 @@ __device__ __forceinline__ void wide_check(const DimArgs& a, const RedState& s, 
       for (int u = 0; u < 4; ++u) {
         code[u] = key[u];
         key[u] = near[u] ? __ldcg(s.r_key + v.toff + slot[u]) : ~0ull;
+        settled += key[u] >= lo && key[u] < hi && (code[u] & 15) < OWN_NONE;
       }
     } else {
       uint64_t h[4];
@@ -928,10 +946,11 @@ __device__ __forceinline__ void wide_check(const DimArgs& a, const RedState& s, 
   }
   const uint64_t un = warp_min_u64(seen.un), ow = warp_min_u64(seen.ow);
   joined = __reduce_add_sync(0xffffffffu, joined);
+  settled = __reduce_add_sync(0xffffffffu, settled);
   if (lane == 0) {
+    wide_count2(&v.c->count, joined, settled);
     if (ow != ~0ull) atomicMin(&v.c->ow, (unsigned long long)ow);
     if (un != ~0ull) atomicMin(&v.c->un, (unsigned long long)un);
-    if (joined) atomicAdd(&v.c->count, joined);
   }
 }
 
@@ -956,7 +975,7 @@ __device__ void wide_process(const DimArgs& a, const RedState& s, const Team& t,
       ents += wide_gen<D>(a, s, w, v, cv, B, lane, ref, kind == REC_PACKED, rank, f, fresh);
     }
   }
-  wide_count_fresh(v.c, lane, fresh);
+  wide_count_fresh(v.c, lane, fresh, (unsigned)ents);
   if (lane == 0 && ents) atomicAdd(s.added, ents);
 }
 
@@ -995,6 +1014,8 @@ __device__ __forceinline__ int wide_begin(const DimArgs& a, const RedState& s, c
     w.j = j;
     w.cl = cl;
     w.step = 0;
+    w.pace = w.each = 0.0f;
+    w.lo = w.hi = 0;
     w.dil = 1;
     w.n[0] = w.n[1] = 0;
     w.tmask = 0;
@@ -1066,10 +1087,15 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
   float again = 0.0f;       // share of a round's rows that come back live in the next one
   uint32_t last = 0;        // rows added last round
   float share = 1.0f;       // of k, to extend the window by
+  const float free = t.size > 1 ? WIDE_TEAM_FREE * (float)t.size : WIDE_FREE;
+  const bool paced = a.amap || (a.opts & RIPS_OPT_NO_APPARENT);  // owners are kept, so that settled rows can be counted
   for (;;) {
     const uint32_t goal = t.size > 1 ? max(w.step / 2, min(max(w.step, WIDE_TEAM_K0), WIDE_TEAM_K1))
                                      : max(w.step / 3, WIDE_K0);
-    const uint32_t k = min(goal, kmax);  // rows with an owner wanted in the window
+    // rows with an owner wanted in the window
+    const float ahead = fmaxf(WIDE_AHEAD * w.pace, free / fmaxf(w.each, 1.0f));
+    const uint32_t k = min(min(goal, kmax), paced ? max((uint32_t)ahead, 2u) : ~0u);
+    const uint32_t crowd = max(2 * k, min(64u, 8 * k));  // and more than these are too many
     const unsigned long long want = max(1ull, min((unsigned long long)((float)k * share) * w.dil, rows));
     bool extend = false;
     uint64_t b = w.bound;
@@ -1127,6 +1153,9 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
     if ((stop & 1u) || w.step > MAX_PIVOT_PASSES) return CH_LONG;
     __syncthreads();
     if (threadIdx.x == 0) {
+      if (w.hi > w.lo) w.pace = 0.5f * (w.pace + (float)w.d.settled);
+      w.lo = w.hi;
+      w.hi = ow == ~0ull ? w.bound : ow;
       if (joined) w.dil = max(1u, joined / max(owned, 1u));
       if (ow == ~0ull) w.n[L_FRONT] = 0;  // no live row: all of them are settled
     }
@@ -1138,13 +1167,13 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
       if (stop & 2u) return CH_HEAVY;
       continue;
     }
-    if (todo > 2 * k && todo > 64) {  // the window's rows have multiplied: keep about the k oldest
+    if (todo > crowd) {  // the window's rows have multiplied: keep about the k oldest
       const uint64_t b2 = min(wide_sample(s, w, p, L_FRONT, k, sm), w.bound);
       if (b2 < w.bound) {
         __syncthreads();
         if (threadIdx.x == 0) w.bound = b2;
         __syncthreads();
-        const int e = wide_split(t, s, w, L_FRONT, b2, L_FRONT, L_MID, ow);
+        const int e = wide_split(t, s, w, L_FRONT, b2, L_FRONT, L_MID, w.lo);
         if (e != CH_DONE) return e;
         if (stop & 2u) return CH_HEAVY;
         share = 0.0f;
@@ -1155,9 +1184,12 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
     } else if (w.n[L_FRONT] > 4 * min((unsigned long long)k * w.dil, rows) + 1024) {  // mostly settled rows: drop them
       const int e = wide_split(t, s, w, L_FRONT, w.bound, L_FRONT, L_MID, ow);
       if (e != CH_DONE) return e;
+      if (threadIdx.x == 0) w.lo = w.hi;  // nothing left to count of this round
+      __syncthreads();
     }
     // the additions, in sections of at most as many rows as the working column leaves room for
     uint32_t grown = 0;
+    float ents = (float)lr;
     for (uint32_t p0 = 0; p0 < todo;) {
       const uint32_t most =
           (uint32_t)min((unsigned long long)(todo - p0), max(64ull, ((unsigned long long)w.used + 65536) >> sbits));
@@ -1166,6 +1198,7 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
       wide_process<D>(a, s, t, w, cv, B, p0, p0 + most);
       if (!wide_sync(t, s, w)) return CH_LONG;
       grown += w.d.add[L_FRONT];
+      ents += (float)w.d.ents;
       p0 += most;
     }
     if (nl) {
@@ -1176,7 +1209,10 @@ __device__ __forceinline__ int wide_advance(const DimArgs& a, const RedState& s,
       if (!wide_sync(t, s, w)) return CH_LONG;
       grown += w.d.add[L_FRONT];
     }
-    if (threadIdx.x == 0) w.step += todo + nl;
+    if (threadIdx.x == 0) {
+      w.each = (w.step ? 0.5f : 1.0f) * ents / (float)(todo + nl) + (w.step ? 0.5f * w.each : 0.0f);
+      w.step += todo + nl;
+    }
     __syncthreads();
     // the rows expected live next time are left out of the next extension
     last = todo + nl;

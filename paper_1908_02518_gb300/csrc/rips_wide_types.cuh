@@ -15,9 +15,11 @@ constexpr int WIDE_SPARES = 4;
 // what a team's threads count during one section (between two team barriers)
 struct WideCount {
   unsigned add[2];  // rows appended to each list
-  unsigned fresh;   // rows entered into the table
+  unsigned fresh;   // rows entered into the table, and
+  unsigned ents;    // entries added (one 64-bit count)
+  unsigned count;   // rows with an owner among those that join the front (or rows of a stored run), and
+  unsigned settled; // owned rows that the round before last settled (one 64-bit count)
   unsigned todo;    // rows put on the work list
-  unsigned count;   // rows with an owner among those that join the front; rows of a stored run
   unsigned nlong;   // stored runs left to the whole team
   unsigned stop;    // 1: out of time, 2: give way to a larger team
   unsigned long long un, ow;   // oldest live row without and with an owner
@@ -36,6 +38,8 @@ struct WideShared {
 // state of a column's reduction, the same in every block of its team
 struct WideState {
   uint32_t j, cl, step, dil;
+  float pace, each;      // owned rows settled a round, entries an added column
+  uint64_t lo, hi;       // oldest live owned row of the last check but one, and of the last
   int ph, tcur;
   uint32_t n[2];
   int cur[2];
