@@ -770,9 +770,10 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       }
     }
     bool done = false;
-    for (int attempt = 0; attempt < 6 && !done; ++attempt) {
-      CR(ensure(w.r_key, rcap * 8));
-      CR(ensure(w.r_coef, rcap * 4));
+    int grid = blocks;
+    for (int attempt = 0; attempt < 16 && !done; ++attempt) {
+      CR(ensure(w.r_key, rcap * 8, false));
+      CR(ensure(w.r_coef, rcap * 4, false));
       w.r_cap = rcap;
       CK(cudaMemsetAsync(w.tkeys[tb].p, 0xFF, (size_t)tcap * 8, s));
       CK(cudaMemsetAsync(w.tvals[tb].p, 0xFF, (size_t)tcap * 4, s));
@@ -810,7 +811,7 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       rs.err = P<uint32_t>(w.err);
       {
         KTimer kt(w, RIPS_K_REDUCE, s);
-        CK(launch_reduction(a, rs, blocks, counts, s));
+        CK(launch_reduction(a, rs, grid, counts, s));
       }
       {
         KTimer kt(w, RIPS_K_READOUT, s);
@@ -826,9 +827,17 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       CR(sync_read(w, s));
       if (int e = map_device_error(hp->u32[8])) return e;  // whatever else failed, with a full arena or not
       if (hp->u32[8] & ERRF_ARENA) {
-        // start this dimension's reduction over with a larger arena (the readout of a failed one writes nothing)
+        // Start this dimension's reduction over (the readout of a failed one writes nothing) in a larger arena, up to
+        // four fifths of the memory there is, and after that with a quarter of the blocks: the tables of the columns
+        // under way, one to a block, are what fills it where columns grow to a good part of all rows (random lengths on
+        // 400 points: 1.8 million rows a column).
         CK(cudaMemsetAsync(w.err.p, 0, 4, s));
-        rcap *= 8;
+        size_t free_b = 0, total_b = 0;
+        CK(cudaMemGetInfo(&free_b, &total_b));
+        const size_t most = (free_b + w.r_key.cap + w.r_coef.cap) / 12 / 5 * 4;
+        if (rcap < most) rcap = std::min(8 * rcap, most);
+        else if (grid > 1) grid = (grid + 3) / 4;
+        else break;
         continue;
       }
       out.stats.resize((size_t)C * (dim_max + 1));
