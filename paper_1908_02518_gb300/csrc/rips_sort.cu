@@ -11,9 +11,10 @@
 //       with equal digits keep their relative order (LSD correctness); the
 //       tile is put in digit order in shared memory and written out in runs.
 // Bits below `low_bit` are not sorted: callers whose keys already come in the
-// order of those bits save their passes.  Bound by L2 and HBM traffic for long
-// inputs (3 x 8 bytes a key and pass: 8.4 million keys 95 us a pass, 140 us when
-// keys were scattered straight from registers after being ranked twice) and by
+// order of those bits save their passes.  Bound, for long inputs, by the ranking in
+// shared memory where many keys share a digit (8.4 million keys: a scatter 73 us, 38
+// where digits are spread, with 3 x 8 bytes a key and pass to move; a pass 95 us, 140
+// when keys were scattered straight from registers after being ranked twice) and by
 // launches for short ones (11000 keys: 0.06 ms in 4 or 5 passes of two launches,
 // 0.14 in 7 of three).  Tiles of 2048 keys give 50 blocks at 100000 keys.
 

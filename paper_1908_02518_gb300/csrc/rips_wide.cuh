@@ -41,8 +41,8 @@
 // (0.5 us in a block, 4 to 8 us over the grid), whatever the number of rows, so
 // the gain is in rows per section.  Reduction before (one addition at a time, 10
 // to 25 us each) and after, GB300: 2,048 rotations, chains of 16,240 and 15,062
-// additions, 319 -> 14 ms; 4,096 rotations, 580,824 and 78,690 additions, 7,328 ->
-// 78 ms; torus of 1,000 points, 730 additions, 11.6 -> 2.1 ms (4 % of the cycles
+// additions, 319 -> 15 ms; 4,096 rotations, 580,824 and 78,690 additions, 7,328 ->
+// 76 ms; torus of 1,000 points, 730 additions, 11.6 -> 2.2 ms (4 % of the cycles
 // issue, warps wait at barriers).
 //
 // A team is one block (counters in shared memory) or several (counters in the
