@@ -828,15 +828,15 @@ int run_batch(Workspace& w, const float* dD, const std::vector<int64_t>& ns, int
       if (int e = map_device_error(hp->u32[8])) return e;  // whatever else failed, with a full arena or not
       if (hp->u32[8] & ERRF_ARENA) {
         // Start this dimension's reduction over (the readout of a failed one writes nothing) in a larger arena, up to
-        // four fifths of the memory there is, and after that with a quarter of the blocks: the tables of the columns
+        // four fifths of the memory there is, and after that with half of the blocks: the tables of the columns
         // under way, one to a block, are what fills it where columns grow to a good part of all rows (random lengths on
-        // 400 points: 1.8 million rows a column).
+        // 400 points; 700 words of 64 bits by Hamming distance: 9 s, 27 with a quarter of the blocks).
         CK(cudaMemsetAsync(w.err.p, 0, 4, s));
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));
         const size_t most = (free_b + w.r_key.cap + w.r_coef.cap) / 12 / 5 * 4;
         if (rcap < most) rcap = std::min(8 * rcap, most);
-        else if (grid > 1) grid = (grid + 3) / 4;
+        else if (grid > 1) grid = (grid + 1) / 2;
         else break;
         continue;
       }
